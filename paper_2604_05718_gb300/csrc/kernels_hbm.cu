@@ -338,14 +338,41 @@ __global__ void compose_kernel(const int32_t* map1, const int64_t* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// Gather reconstruction (Eq. 4), a pure copy.  A warp takes 32 consecutive
-// grid rows: lane l resolves row p0 + l (its image, its map entry and the
-// source row, all independent loads across the lanes), then the warp copies
-// the rows RG at a time with every lane moving 16-byte vectors.  With
-// COMPOSE the source is composed on the way (Eq. 3):
-// r*(p) = map2[off1_b + map1[p]], and r* is written to out_map if given.
+// Gather reconstruction (Eq. 4), a pure copy.  A warp takes `per_warp` (at
+// most kGatherRows) consecutive grid rows: lane l resolves row p0 + l (its
+// image, its map entry and the source row, all independent loads across the
+// lanes), then the warp copies the rows as one run of 16-byte vectors, U of
+// them in flight per lane whatever the row length.  With COMPOSE the source
+// is composed on the way (Eq. 3): r*(p) = map2[off1_b + map1[p]], and r* is
+// written to out_map if given.
+//
+// Large grids are bound by HBM, small ones by the chain of dependent loads
+// (offsets, maps, row), so the rows are dealt evenly over the whole GPU: 32
+// rows a warp, four at a time, left 1024 rows of 768 bf16 on 32 warps (10.0
+// us, now 1.4) and 36864 rows of 1024 on 1152 warps (24.5 us, now 15.7).
+// Runs of 8 rows with 12 vectors in flight were the fastest on 65536 rows of
+// 768 bf16 (whole step 202.4 us; 4 rows and 8 vectors 203.3, up to 32 rows
+// and 8 vectors 203.6).
 // ---------------------------------------------------------------------------
-template <int U, int RG, bool COMPOSE>
+constexpr int kGatherVecs = 12;
+constexpr int kGatherRows = 8;
+static_assert(kGatherRows <= 32, "one lane resolves each row of a run");
+
+// Quotient e / nvec for 0 <= e < 2^17 and 1 <= nvec <= 2^12 (rows of at most
+// 64 KiB): magic = floor(2^31 / nvec) + 1, so the quotient is off by less than
+// e / 2^31 < 1 / nvec.
+struct RowDiv {
+  uint32_t nvec, magic;
+  __device__ __forceinline__ uint32_t operator()(uint32_t e) const {
+    return static_cast<uint32_t>((static_cast<uint64_t>(e) * magic) >> 31);
+  }
+};
+RowDiv row_div(int row_bytes) {
+  const uint32_t nvec = static_cast<uint32_t>(row_bytes >> 4);
+  return {nvec, nvec == 1 ? 0x80000000u : 0x80000000u / nvec + 1u};
+}
+
+template <int U, bool COMPOSE>
 __global__ void __launch_bounds__(kThreads) gather_kernel(const uint8_t* __restrict__ merged,
                                                           const int64_t* __restrict__ moff,
                                                           int64_t merged_rows,
@@ -354,25 +381,27 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const uint8_t* __restr
                                                           int64_t grid_rows,
                                                           const int32_t* __restrict__ map2,
                                                           const int64_t* __restrict__ off1, int64_t rows1,
-                                                          int32_t* out_map, int batch, int row_bytes,
+                                                          int32_t* out_map, int batch, RowDiv row, int per_warp,
                                                           uint8_t* __restrict__ out, int32_t* status) {
   MPM_TRACE_BEGIN(MPM_TRACE_GATHER);
   wait_for_previous_grid();
   MPM_TRACE_WAITED();
   const int lane = threadIdx.x & 31;
-  const int64_t warp = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
+  // Neighbouring runs go to neighbouring blocks, so that few rows still use
+  // every SM.
+  const int64_t warp = static_cast<int64_t>(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
   const int64_t used = clamp64(goff[batch], 0, grid_rows);
-  const int nvec = row_bytes >> 4;
   ImageCursor cur;
-  for (int64_t p0 = warp * 32; p0 < used; p0 += nwarps * 32) {
+  for (int64_t p0 = warp * per_warp; p0 < used; p0 += nwarps * per_warp) {
     // Lane l resolves grid row p0 + l.
     const int64_t p = p0 + lane;
-    int64_t src = -1;  // merged row to copy, -1 = none (zero row)
-    if (p < used) {
+    const int nrows = static_cast<int>(used - p0 < per_warp ? used - p0 : per_warp);
+    int32_t src = -1;  // merged row to copy, -1 = none (zero row)
+    if (lane < nrows) {
+      int32_t m = map[p];
       cur.locate(goff, batch, p);
       const int64_t mlo = __ldg(moff + cur.b), mhi = __ldg(moff + cur.b + 1);
-      int32_t m = map[p];
       bool ok = p >= cur.lo && p < cur.hi;
       if (COMPOSE) {
         // Stage-1 index of this grid row, then its stage-2 (merged) index.
@@ -384,38 +413,44 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const uint8_t* __restr
       if (!ok) report(status, MPM_ERR_DEVICE_CHECK, static_cast<int32_t>(p));
       // This lane alone reads and writes entry p, so out_map may alias map.
       if (COMPOSE && out_map != nullptr) out_map[p] = ok ? m : -1;
-      src = ok ? mlo + m : -1;
+      src = ok ? static_cast<int32_t>(mlo + m) : -1;
     }
-    const int nrows = static_cast<int>(used - p0 < 32 ? used - p0 : 32);
-    for (int r0 = 0; r0 < nrows; r0 += RG) {
-      int64_t s[RG];
+    const uint32_t total = static_cast<uint32_t>(nrows) * row.nvec;
+    uint4* dst = reinterpret_cast<uint4*>(out) + p0 * row.nvec;
+    for (uint32_t e0 = lane; e0 < total + lane; e0 += 32 * U) {
+      uint4 val[U];
 #pragma unroll
-      for (int g = 0; g < RG; ++g) s[g] = __shfl_sync(0xFFFFFFFFu, src, (r0 + g) & 31);
-      for (int v0 = lane; v0 < nvec; v0 += 32 * U) {
-        uint4 val[RG][U];
-#pragma unroll
-        for (int g = 0; g < RG; ++g)
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int v = v0 + 32 * u;
-            if (r0 + g < nrows && v < nvec)
-              val[g][u] = s[g] >= 0 ? __ldg(reinterpret_cast<const uint4*>(merged + s[g] * row_bytes) + v)
-                                    : make_uint4(0, 0, 0, 0);
-          }
-#pragma unroll
-        for (int g = 0; g < RG; ++g)
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int v = v0 + 32 * u;
-            if (r0 + g < nrows && v < nvec)
-              __stcs(reinterpret_cast<uint4*>(out + (p0 + r0 + g) * row_bytes) + v, val[g][u]);
-          }
+      for (int u = 0; u < U; ++u) {
+        const uint32_t e = e0 + 32 * u;
+        const uint32_t r = row(e);
+        const int32_t s = __shfl_sync(0xFFFFFFFFu, src, r & 31);
+        if (e < total)
+          val[u] = s >= 0 ? __ldg(reinterpret_cast<const uint4*>(merged) + static_cast<int64_t>(s) * row.nvec +
+                                  (e - r * row.nvec))
+                          : make_uint4(0, 0, 0, 0);
       }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (e0 + 32 * u < total) __stcs(dst + e0 + 32 * u, val[u]);
     }
   }
 }
 
 int grid_for(int num_sms, int per_sm) { return (num_sms > 0 ? num_sms : 1) * per_sm; }
+
+// Blocks and rows per warp of the gather for `rows` grid rows: at most one
+// wave of blocks, and rows dealt evenly over its warps (at most kGatherRows a
+// warp and round).
+struct GatherShape {
+  int grid, per_warp;
+};
+GatherShape gather_shape(int64_t rows, int wave) {
+  const int64_t warps = static_cast<int64_t>(wave) * (kThreads / 32);
+  const int64_t rounds = (rows + kGatherRows * warps - 1) / (kGatherRows * warps);
+  const int64_t per_warp = (rows + warps * rounds - 1) / (warps * rounds);
+  const int64_t need = (rows + per_warp * (kThreads / 32) - 1) / (per_warp * (kThreads / 32));
+  return {static_cast<int>(need < wave ? need : wave), static_cast<int>(per_warp)};
+}
 
 }  // namespace
 
@@ -472,11 +507,13 @@ cudaError_t launch_gather(const void* merged, const int64_t* moff, int64_t merge
                           int dim, bool bf16, void* out, int32_t* status, int num_sms,
                           cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
-  static const int per_sm = resident_per_sm(gather_kernel<3, 4, false>, kThreads, 8);
-  return launch_dependent(gather_kernel<3, 4, false>, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
-                          static_cast<const uint8_t*>(merged), moff, merged_rows, map, goff, grid_rows,
-                          static_cast<const int32_t*>(nullptr), static_cast<const int64_t*>(nullptr),
-                          static_cast<int64_t>(0), static_cast<int32_t*>(nullptr), batch, row_bytes,
+  auto kernel = gather_kernel<kGatherVecs, false>;
+  static const int per_sm = resident_per_sm(kernel, kThreads, 8);
+  const GatherShape g = gather_shape(grid_rows, grid_for(num_sms, per_sm));
+  return launch_dependent(kernel, dim3(g.grid), dim3(kThreads), 0, stream, static_cast<const uint8_t*>(merged), moff,
+                          merged_rows, map, goff, grid_rows, static_cast<const int32_t*>(nullptr),
+                          static_cast<const int64_t*>(nullptr), static_cast<int64_t>(0),
+                          static_cast<int32_t*>(nullptr), batch, row_div(row_bytes), g.per_warp,
                           static_cast<uint8_t*>(out), status);
 }
 
@@ -486,10 +523,12 @@ cudaError_t launch_compose_gather(const void* merged, const int64_t* moff, int64
                                   bool bf16, void* out, int32_t* out_map, int32_t* status, int num_sms,
                                   cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
-  static const int per_sm = resident_per_sm(gather_kernel<3, 4, true>, kThreads, 8);
-  return launch_dependent(gather_kernel<3, 4, true>, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
-                          static_cast<const uint8_t*>(merged), moff, merged_rows, map1, off0, rows0, map2, off1,
-                          rows1, out_map, batch, row_bytes, static_cast<uint8_t*>(out), status);
+  auto kernel = gather_kernel<kGatherVecs, true>;
+  static const int per_sm = resident_per_sm(kernel, kThreads, 8);
+  const GatherShape g = gather_shape(rows0, grid_for(num_sms, per_sm));
+  return launch_dependent(kernel, dim3(g.grid), dim3(kThreads), 0, stream, static_cast<const uint8_t*>(merged), moff,
+                          merged_rows, map1, off0, rows0, map2, off1, rows1, out_map, batch, row_div(row_bytes),
+                          g.per_warp, static_cast<uint8_t*>(out), status);
 }
 
 }  // namespace mpm
