@@ -66,8 +66,8 @@ cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, in
 AffinityTile pair_tile();
 
 // Mutual check, representative scan, per-image counts, output offsets.
-cudaError_t launch_mutual_compact(int batch, int64_t chunk, const Workspace& ws, int32_t* out_map,
-                                  int64_t* out_offsets, cudaStream_t stream);
+cudaError_t launch_mutual_compact(int batch, int64_t rows, int64_t chunk, const Workspace& ws, int32_t* out_map,
+                                  int64_t* out_offsets, int num_sms, cudaStream_t stream);
 
 // Pair average + compaction into the packed output.
 cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch, int64_t rows,

@@ -243,7 +243,7 @@ mpm_status merge_impl(const void* tokens, const int64_t* offsets, int32_t batch,
   if (!mark(3) || !mark(4)) return MPM_ERR_CUDA;
   {
     const Range r("mpm.mutual_scan");
-    e = mpm::launch_mutual_compact(batch, chunk, ws, out_map, out_offsets, s);
+    e = mpm::launch_mutual_compact(batch, rows, chunk, ws, out_map, out_offsets, sms, s);
   }
   if (e != cudaSuccess || !mark(5) || !mark(6)) return MPM_ERR_CUDA;
   if (rows > 0) {
