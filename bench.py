@@ -320,11 +320,6 @@ def traffic_for(kernel_files, rows_per_launch: float):
 # ---------------------------------------------------------------------------
 # The GPU path
 # ---------------------------------------------------------------------------
-# Nominal dense tf32 / bf16 tensor throughput (1.1 / 2.25 PFLOP/s per GB300):
-# the fp32 path's peak is the measured bf16 peak times this ratio.
-TF32_PER_BF16 = 1.1 / 2.25
-
-
 def new_events(stream, n):
     """n timing events, recorded once so that their CUDA handles exist."""
     import torch
@@ -488,9 +483,9 @@ def step_metrics(p: Step, t: dict, peaks: dict, peak_kind: str) -> dict:
     aff_ms = t["aff_ms_1"] + t["aff_ms_2"]
     aff_flops = [alg1] * len(t["aff_ms_1"]) + [alg2] * len(t["aff_ms_2"])
     achieved = sum(aff_flops) / (sum(aff_ms) * 1e-3) / 1e12
-    ratio = 1.0 if cfg.dtype == "bf16" else TF32_PER_BF16
-    burst = ratio * peaks.get("bf16_tflops", FALLBACK_PEAKS["bf16_tflops"])
-    sustained = ratio * peaks.get("bf16_tflops_sustained", FALLBACK_PEAKS["bf16_tflops_sustained"])
+    # fp32 tokens run three fp16 products per term, at the bf16 rate.
+    burst = peaks.get("bf16_tflops", FALLBACK_PEAKS["bf16_tflops"])
+    sustained = peaks.get("bf16_tflops_sustained", FALLBACK_PEAKS["bf16_tflops_sustained"])
     # What the tensor pipe executes (bf16): the 256 x 256 tiles on or above
     # each image's diagonal, over K padded to 16 (the MMA's K).  The R tiles
     # of an image's last column block are narrow (256 x 128) when that block
@@ -560,7 +555,7 @@ def workload_summary(p: Step, t: dict, m: dict) -> dict:
         "affinity_frac_of_burst": m["aff_tflops"] / m["aff_peak_burst"],
         "affinity_frac_of_sustained": m["aff_tflops"] / m["aff_peak_sustained"],
         "affinity_peak": ("bf16 dense" if p.cfg.dtype == "bf16" else
-                          "tf32 dense = bf16 x 1.1/2.25 (nominal ratio); three tf32 products per term"),
+                          "fp16 dense (the bf16 rate); three fp16 products per term"),
         "affinity_us": {k: v for k, v in t["kern"].items() if k.startswith("affinity")},
         "pipeline_frac": m["pipeline"]["frac"],
     }
@@ -742,7 +737,7 @@ def run_mpm(args):
             "merged_tokens_full": res[0][1], "merged_tokens_chunk_1024": res[1024][1],
         }
 
-    # ---------------- fp32 tokens: three tf32 products on the tensor cores vs CUDA-core FMA ----------------
+    # ---------------- fp32 tokens: three fp16 products on the tensor cores vs CUDA-core FMA ----------------
     # The nearest-neighbour step (Eq. 1 + arg max) of the same image shapes
     # in fp32, through MPM_NN_TCGEN05_PAIR (the fp32 default) and MPM_NN_SIMT.
     fp32 = None
@@ -770,7 +765,7 @@ def run_mpm(args):
             f_nn[algo] = nn_f
         fp32 = {
             "workload": f"{f_cfg.batch} x {int(fb.offsets[1])} tokens x {f_cfg.dim} fp32 (vit_b shapes)",
-            "nn_us_tensor_3xtf32": f_us["tcgen05_pair"], "nn_us_simt_fma": f_us["simt"],
+            "nn_us_tensor_3xf16": f_us["tcgen05_pair"], "nn_us_simt_fma": f_us["simt"],
             "speedup": f_us["simt"] / f_us["tcgen05_pair"],
             "same_neighbour_frac": float((f_nn["tcgen05_pair"] == f_nn["simt"]).float().mean()),
         }

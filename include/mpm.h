@@ -80,8 +80,9 @@ typedef enum mpm_nn_algo {
                               feeding both its rows and its columns (bf16) */
   MPM_NN_TCGEN05_PAIR = 4  /* symmetric, 256 x 256 tiles on SM pairs with
                               tcgen05.mma.cta_group::2: bf16 products for bf16
-                              tokens; for fp32 tokens three tf32 products per
-                              term (x = hi + lo with hi the tf32 rounding of x:
+                              tokens; for fp32 tokens three fp16 products per
+                              term (a row's values scaled by one power of two,
+                              x = hi + lo with hi the fp16 rounding of x:
                               hi.hi + hi.lo + lo.hi, accumulated in fp32) */
 } mpm_nn_algo;
 
@@ -97,7 +98,7 @@ MPM_API const char* mpm_status_string(mpm_status status);
  * The workspace must be 256-byte aligned.  It holds per-row inverse norms,
  * packed arg-max keys, the representative list, per-image counts, sanitised
  * offsets, the work plan and the device status word; for fp32 tokens also
- * the tf32 high and low parts of the tokens (2 * rows * dim floats).
+ * room for the high and low parts of the tokens (2 * rows * dim floats).
  */
 MPM_API size_t mpm_merge_workspace_size(int64_t rows, int32_t batch, int32_t dim, mpm_dtype dtype);
 
@@ -156,7 +157,7 @@ MPM_API mpm_status mpm_merge_timed(const void* tokens, const int64_t* offsets, i
  *    mpm_merge_workspace_size(rows, batch, dim, dtype) exceeds
  *    MPM_NO_ALLOC_SCRATCH_BYTES (8 MiB), and allocates nothing in any case.
  *    The workspace takes about 20 bytes per row for bf16 tokens, so 8 MiB
- *    holds about 400,000 rows; for fp32 tokens it also holds the two tf32
+ *    holds about 400,000 rows; for fp32 tokens it also holds room for two
  *    split copies of the tokens, 20 + 8 * dim bytes per row: about 5,400
  *    rows at dim 192 and 1,360 rows at dim 768.  (Plus 20 bytes per image
  *    and up to 256 bytes of alignment per region either way.)

@@ -13,10 +13,13 @@
 //    KiB per stage instead of 96 KiB, which leaves room for three stages and
 //    cuts the shared-memory traffic of the tensor cores by a third.
 //  * bf16 tokens: a stage holds 128 features (two 64-feature TMA boxes per
-//    operand) and takes eight K = 16 MMAs.  fp32 tokens (TF32 = true): every
-//    value is split as x = hi + lo (hi the tf32 rounding of x, written with
-//    lo by the prep kernel), a stage holds 32 features of A hi, A lo, B hi
-//    and B lo, and takes twelve K = 8 tf32 MMAs: hi.hi + hi.lo + lo.hi.
+//    operand) and takes eight K = 16 MMAs.  fp32 tokens (SPLIT = true): every
+//    row is scaled by a power of two and its values split into fp16 parts,
+//    x = hi + lo (written by the prep kernel); a stage holds 64 features of A
+//    hi, A lo, B hi and B lo, and takes twelve K = 16 fp16 MMAs: hi.hi +
+//    hi.lo + lo.hi.  (Three tf32 products, of parts with as many bits, ran
+//    at half the rate and moved twice the bytes: 177.6 instead of 100.1 us
+//    for 64 x 1024 x 768.)
 //    The MMA warp issues a whole stage and its release commit from one asm
 //    block: its sub-partition also runs two epilogue warps, and every
 //    instruction it saves per stage keeps the tensor core fed.
@@ -97,14 +100,13 @@ constexpr uint32_t IDESC = ptx::idesc_bf16_f32(2 * HALF, TILE);
 // Narrow tiles (at most HALF columns of the tile inside the chunk) run
 // N = HALF MMAs: half the tensor work, and each CTA holds HALF / 2 B rows.
 constexpr uint32_t IDESC_NARROW = ptx::idesc_bf16_f32(2 * HALF, HALF);
-// fp32 tokens: three tf32 products per K slice (hi hi + hi lo + lo hi, the
-// "3xTF32" split), with a stage of 32 features holding four 16 KiB slices:
-// A high, A low, B high, B low (one 128-byte swizzle row of fp32 each).
-constexpr int TF_BOX_K = 32;
-constexpr int TF_BK = TF_BOX_K;
-constexpr uint32_t IDESC_TF32 = ptx::idesc_tf32_f32(2 * HALF, TILE);
-constexpr uint32_t IDESC_TF32_NARROW = ptx::idesc_tf32_f32(2 * HALF, HALF);
-static_assert(4 * ATOM_BYTES == STAGE_BYTES && HALF * TF_BOX_K * 4 == ATOM_BYTES, "same stage size for both paths");
+// fp32 tokens: three fp16 products per K slice (hi hi + hi lo + lo hi), with
+// a stage of 64 features holding four 16 KiB slices: A high, A low, B high, B
+// low (one 128-byte swizzle row of fp16 each).
+constexpr int SPLIT_BK = BOX_K;
+constexpr uint32_t IDESC_SPLIT = ptx::idesc_f16_f32(2 * HALF, TILE);
+constexpr uint32_t IDESC_SPLIT_NARROW = ptx::idesc_f16_f32(2 * HALF, HALF);
+static_assert(4 * ATOM_BYTES == STAGE_BYTES, "same stage size for both paths");
 constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;
 constexpr int kMaxItems = 160;
 constexpr int kMaxStagedImages = 511;  // plan and offsets staged in shared memory up to this batch
@@ -280,46 +282,35 @@ __device__ __forceinline__ void mma_stage_full(uint32_t d_tmem, uint64_t a_desc,
       : "memory");
 }
 
-// The twelve MMAs of one full fp32 stage (32 features = four K = 8 slices of
-// 32 bytes), three tf32 products per slice, then the release commit.  The
+// The twelve MMAs of one full fp32 stage (64 features = four K = 16 slices of
+// 32 bytes), three fp16 products per slice, then the release commit.  The
 // stage's slices lie at a_desc (A high), +1024 (A low), +2048 (B high) and
 // +3072 (B low) in descriptor units of 16 bytes.
-__device__ __forceinline__ void mma_stage_tf32x3(uint32_t d_tmem, uint64_t a_desc, uint32_t idesc,
+__device__ __forceinline__ void mma_stage_split(uint32_t d_tmem, uint64_t a_desc, uint32_t idesc,
                                                  uint32_t accumulate, uint64_t* release) {
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t.reg .b64 ah, al, bh, bl;\n\t"
       "setp.ne.b32 p, %3, 0;\n\t"
       "setp.ne.b32 q, %5, 0;\n\t"
       "add.s64 al, %1, 1024;\n\tadd.s64 bh, %1, 2048;\n\tadd.s64 bl, %1, 3072;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, bh, %2, p;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, bl, %2, q;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], al, bh, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, bh, %2, p;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, bl, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
       "add.s64 ah, %1, 2;\n\tadd.s64 al, %1, 1026;\n\tadd.s64 bh, %1, 2050;\n\tadd.s64 bl, %1, 3074;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], ah, bh, %2, q;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], ah, bl, %2, q;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], al, bh, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bl, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
       "add.s64 ah, %1, 4;\n\tadd.s64 al, %1, 1028;\n\tadd.s64 bh, %1, 2052;\n\tadd.s64 bl, %1, 3076;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], ah, bh, %2, q;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], ah, bl, %2, q;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], al, bh, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bl, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
       "add.s64 ah, %1, 6;\n\tadd.s64 al, %1, 1030;\n\tadd.s64 bh, %1, 2054;\n\tadd.s64 bl, %1, 3078;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], ah, bh, %2, q;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], ah, bl, %2, q;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], al, bh, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bl, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%4], %6;\n\t}"
       ::"r"(d_tmem), "l"(a_desc), "r"(idesc), "r"(accumulate), "r"(ptx::smem_addr(release)), "r"(1u),
       "h"(static_cast<uint16_t>(3))
-      : "memory");
-}
-
-// One tf32 MMA (K = 8), issued by one thread.
-__device__ __forceinline__ void mma_pair_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                              uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -349,14 +340,14 @@ __device__ __noinline__ void mma_partial_stage_bf16(uint32_t d_tmem, uint64_t a_
   }
   commit_both(release);
 }
-__device__ __noinline__ void mma_partial_stage_tf32(uint32_t d_tmem, uint64_t a_desc, uint32_t idesc, int kb,
+__device__ __noinline__ void mma_partial_stage_split(uint32_t d_tmem, uint64_t a_desc, uint32_t idesc, int kb,
                                                     int dim, uint64_t* release) {
-  for (int kk = 0; kk < TF_BK / 8 && kb * TF_BK + kk * 8 < dim; ++kk) {
+  for (int kk = 0; kk < SPLIT_BK / 16 && kb * SPLIT_BK + kk * 16 < dim; ++kk) {
     const uint64_t ah = a_desc + 2 * kk, al = ah + (ATOM_BYTES >> 4);
     const uint64_t bh = ah + 2 * (ATOM_BYTES >> 4), bl = ah + 3 * (ATOM_BYTES >> 4);
-    mma_pair_tf32(d_tmem, ah, bh, idesc, (kb | kk) != 0 ? 1u : 0u);
-    mma_pair_tf32(d_tmem, ah, bl, idesc, 1u);
-    mma_pair_tf32(d_tmem, al, bh, idesc, 1u);
+    mma_pair(d_tmem, ah, bh, idesc, (kb | kk) != 0 ? 1u : 0u);
+    mma_pair(d_tmem, ah, bl, idesc, 1u);
+    mma_pair(d_tmem, al, bh, idesc, 1u);
   }
   commit_both(release);
 }
@@ -378,13 +369,13 @@ __device__ __forceinline__ void fail(Control* ctl, int32_t* status, int32_t role
   report(status, MPM_ERR_DEVICE_TIMEOUT, role);
 }
 
-// TF32: fp32 tokens through the three-product tf32 split (tmap = high
-// parts, tmap_lo = low parts); otherwise bf16 tokens (tmap_lo unused).
-template <bool TF32, int EPIW>
+// SPLIT: fp32 tokens through three fp16 products (tmap = high parts, tmap_lo =
+// low parts); otherwise bf16 tokens (tmap_lo unused).
+template <bool SPLIT, int EPIW>
 __global__ void __launch_bounds__(Epi<EPIW>::THREADS, 1)
     affinity_pair_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_lo,
                          int batch, int dim, int64_t chunk, Workspace ws) {
-  constexpr int kBK = TF32 ? TF_BK : BK;
+  constexpr int kBK = SPLIT ? SPLIT_BK : BK;
   constexpr int EPI_WARPS = Epi<EPIW>::WARPS;
   constexpr int EPI_COLS = Epi<EPIW>::COLS;
   constexpr int THREADS = Epi<EPIW>::THREADS;
@@ -496,7 +487,7 @@ __global__ void __launch_bounds__(Epi<EPIW>::THREADS, 1)
           uint8_t* sa = stages + stage * STAGE_BYTES;
           const uint32_t full_leader = map_to_rank(ptx::smem_addr(&ctl->full[stage]), 0);
           if (leader) ptx::mbar_arrive_expect_tx(&ctl->full[stage], 2 * STAGE_BYTES);
-          if constexpr (TF32) {
+          if constexpr (SPLIT) {
             tma_load_2d_pair(sa, &tmap, full_leader, kb * kBK, arow);                    // A high
             tma_load_2d_pair(sa + ATOM_BYTES, &tmap_lo, full_leader, kb * kBK, arow);    // A low
             tma_load_2d_pair(sa + 2 * ATOM_BYTES, &tmap, full_leader, kb * kBK, brow);   // B high
@@ -542,11 +533,11 @@ __global__ void __launch_bounds__(Epi<EPIW>::THREADS, 1)
                                           : is_narrow(decode_item_slow(plan, soff, batch, cid + k * clusters, chunk,
                                                                        split_from));
         // One tile's stages, with its instruction descriptors as compile-time
-        // constants (ID, ID_TF32): the tile shape is chosen once per tile,
+        // constants (ID, ID_SPLIT): the tile shape is chosen once per tile,
         // outside the stage loop, so no descriptor is a run-time value.
-        auto issue_tile = [&](auto id, auto id_tf32) {
+        auto issue_tile = [&](auto id, auto id_split) {
           [[maybe_unused]] constexpr uint32_t ID = decltype(id)::value;            // bf16 instances
-          [[maybe_unused]] constexpr uint32_t ID_TF32 = decltype(id_tf32)::value;  // tf32 instance
+          [[maybe_unused]] constexpr uint32_t ID_SPLIT = decltype(id_split)::value;  // split instance
           for (int kb = 0; kb < ksteps; ++kb) {
             if (!ptx::mbar_wait(&ctl->full[stage], phase, abort_flag, WAIT_LIMIT_NS)) {
               fail(ctl, ws.status, 13);
@@ -555,11 +546,11 @@ __global__ void __launch_bounds__(Epi<EPIW>::THREADS, 1)
             }
             ptx::tc_fence_after_sync();
             const uint64_t a_desc = desc0 + static_cast<uint64_t>((stage * STAGE_BYTES) >> 4);
-            if constexpr (TF32) {
+            if constexpr (SPLIT) {
               if ((kb + 1) * kBK <= dim) {
-                mma_stage_tf32x3(d_tmem, a_desc, ID_TF32, kb != 0 ? 1u : 0u, &ctl->empty[stage]);
+                mma_stage_split(d_tmem, a_desc, ID_SPLIT, kb != 0 ? 1u : 0u, &ctl->empty[stage]);
               } else {
-                mma_partial_stage_tf32(d_tmem, a_desc, ID_TF32, kb, dim, &ctl->empty[stage]);
+                mma_partial_stage_split(d_tmem, a_desc, ID_SPLIT, kb, dim, &ctl->empty[stage]);
               }
             } else if ((kb + 1) * BK <= dim) {
               mma_stage_full(d_tmem, a_desc, ID, kb != 0 ? 1u : 0u, &ctl->empty[stage]);
@@ -573,13 +564,13 @@ __global__ void __launch_bounds__(Epi<EPIW>::THREADS, 1)
           }
         };
         using NarrowId = std::integral_constant<uint32_t, IDESC_NARROW>;
-        using NarrowIdTf32 = std::integral_constant<uint32_t, IDESC_TF32_NARROW>;
+        using NarrowIdSplit = std::integral_constant<uint32_t, IDESC_SPLIT_NARROW>;
         using FullId = std::integral_constant<uint32_t, IDESC>;
-        using FullIdTf32 = std::integral_constant<uint32_t, IDESC_TF32>;
+        using FullIdSplit = std::integral_constant<uint32_t, IDESC_SPLIT>;
         if (narrow)
-          issue_tile(NarrowId{}, NarrowIdTf32{});
+          issue_tile(NarrowId{}, NarrowIdSplit{});
         else
-          issue_tile(FullId{}, FullIdTf32{});
+          issue_tile(FullId{}, FullIdSplit{});
         if (!ok) break;
         commit_both(&ctl->acc_full[acc]);
         if (++acc == 2) {
@@ -723,20 +714,19 @@ cudaError_t trace_copy_pair(unsigned long long* out, bool reset) { return trace_
 
 AffinityTile pair_tile() { return {TILE, TILE, AffinityTile::kUpperSquare}; }
 
-cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, int dim, bool tf32, int64_t chunk,
+cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, int dim, bool split, int64_t chunk,
                                  const Workspace& ws, int num_sms, cudaStream_t stream) {
   PFN_cuTensorMapEncodeTiled_v12000 encode = encoder();
   if (encode == nullptr) return cudaErrorNotSupported;
-  // bf16: the tokens themselves; fp32: the tf32 high and low copies that the
+  // bf16: the tokens themselves; fp32: the fp16 high and low parts that the
   // prep kernel wrote into the workspace.
-  const int esize = tf32 ? 4 : 2;
   const cuuint64_t gdim[2] = {static_cast<cuuint64_t>(dim), static_cast<cuuint64_t>(rows)};
-  const cuuint64_t gstride[1] = {static_cast<cuuint64_t>(dim) * esize};
-  const cuuint32_t box[2] = {static_cast<cuuint32_t>(tf32 ? TF_BOX_K : BOX_K), HALF};
+  const cuuint64_t gstride[1] = {static_cast<cuuint64_t>(split ? split_stride(dim) : dim) * 2};
+  const cuuint32_t box[2] = {BOX_K, HALF};
   const cuuint32_t estride[2] = {1, 1};
-  const CUtensorMapDataType type = tf32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  void* hi = tf32 ? static_cast<void*>(ws.split_hi) : const_cast<void*>(tokens);
-  void* lo = tf32 ? static_cast<void*>(ws.split_lo) : const_cast<void*>(tokens);
+  const CUtensorMapDataType type = split ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  void* hi = split ? static_cast<void*>(ws.split_hi) : const_cast<void*>(tokens);
+  void* lo = split ? static_cast<void*>(ws.split_lo) : const_cast<void*>(tokens);
   if (hi == nullptr || lo == nullptr) return cudaErrorInvalidValue;
   CUtensorMap map, map_lo;
   if (encode(&map, type, 2, hi, gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -753,7 +743,7 @@ cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, in
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const uint64_t bit = 1ull << (dev & 63);
-  const int inst = tf32 ? 0 : (dim <= kWideEpilogueMaxDim ? 2 : 1);
+  const int inst = split ? 0 : (dim <= kWideEpilogueMaxDim ? 2 : 1);
   void (*const kernels[3])(CUtensorMap, CUtensorMap, int, int, int64_t, Workspace) = {
       affinity_pair_kernel<true, 8>, affinity_pair_kernel<false, 8>, affinity_pair_kernel<false, 16>};
   const size_t smem[3] = {smem_bytes<8>(), smem_bytes<8>(), smem_bytes<16>()};

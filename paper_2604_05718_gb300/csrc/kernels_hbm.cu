@@ -36,9 +36,54 @@ struct ImageCursor {
 // Prep: status reset, offsets sanitisation + work plan (block 0), inverse
 // row norms and key reset (all blocks).
 // ---------------------------------------------------------------------------
-// SPLIT: also write the tf32 high / low parts of fp32 tokens (ws.split_hi /
-// split_lo) for the three-product tensor-core path.
-template <bool SPLIT>
+__device__ __forceinline__ void write_plan(const int64_t* __restrict__ offsets, int batch, int64_t rows,
+                                           const AffinityTile& tile, const Workspace& ws) {
+  __shared__ int64_t sh[32];
+  __shared__ int bad;
+  if (threadIdx.x == 0) {
+    ws.status[0] = 0;
+    ws.status[1] = 0;
+    ws.status[2] = 0;
+    bad = -1;
+  }
+  __syncthreads();
+  // soff[b] = min(rows, max_{b' <= b} max(off[b'], 0)): non-decreasing and
+  // in range whatever the caller passed; violations are reported.
+  int64_t carry = 0;
+  for (int base = 0; base <= batch; base += kThreads) {
+    const int idx = base + threadIdx.x;
+    int64_t raw = 0, prev = 0;
+    if (idx <= batch) {
+      raw = offsets[idx];
+      prev = idx > 0 ? offsets[idx - 1] : 0;
+      if ((idx == 0 && raw != 0) || raw < prev || raw > rows) atomicCAS(&bad, -1, idx);
+    }
+    int64_t v = idx <= batch ? clamp64(raw, 0, rows) : 0;
+    int64_t total;
+    int64_t m = block_incl_max<int64_t>(v, sh, &total, 0);
+    m = m > carry ? m : carry;
+    if (idx <= batch) ws.soff[idx] = m;
+    carry = total > carry ? total : carry;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && bad >= 0) report(ws.status, MPM_ERR_DEVICE_CHECK, bad);
+  // plan[b] = number of affinity tiles of the images before b.
+  __threadfence_block();
+  int64_t acc = 0;
+  for (int base = 0; base <= batch; base += kThreads) {
+    const int idx = base + threadIdx.x;
+    int64_t items = 0;
+    if (idx < batch) {
+      const int64_t n = ws.soff[idx + 1] - ws.soff[idx];
+      items = image_items(n, tile);
+    }
+    int64_t total;
+    const int64_t incl = block_incl_sum<int64_t>(items, sh, &total);
+    if (idx <= batch) ws.plan[idx] = acc + incl - items;
+    acc += total;
+  }
+}
+
 __global__ void __launch_bounds__(kThreads) prep_kernel(const uint8_t* __restrict__ tokens,
                                                         const int64_t* __restrict__ offsets,
                                                         int batch, int64_t rows, int row_bytes,
@@ -52,52 +97,7 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const uint8_t* __restric
   // (The other kernels do not trigger early: blocks of a dependent grid
   // parked on SMs were measured to slow the bandwidth-bound kernels.)
   allow_next_grid();
-  if (blockIdx.x == 0) {
-    __shared__ int64_t sh[32];
-    __shared__ int bad;
-    if (threadIdx.x == 0) {
-      ws.status[0] = 0;
-      ws.status[1] = 0;
-      ws.status[2] = 0;
-      bad = -1;
-    }
-    __syncthreads();
-    // soff[b] = min(rows, max_{b' <= b} max(off[b'], 0)): non-decreasing and
-    // in range whatever the caller passed; violations are reported.
-    int64_t carry = 0;
-    for (int base = 0; base <= batch; base += kThreads) {
-      const int idx = base + threadIdx.x;
-      int64_t raw = 0, prev = 0;
-      if (idx <= batch) {
-        raw = offsets[idx];
-        prev = idx > 0 ? offsets[idx - 1] : 0;
-        if ((idx == 0 && raw != 0) || raw < prev || raw > rows) atomicCAS(&bad, -1, idx);
-      }
-      int64_t v = idx <= batch ? clamp64(raw, 0, rows) : 0;
-      int64_t total;
-      int64_t m = block_incl_max<int64_t>(v, sh, &total, 0);
-      m = m > carry ? m : carry;
-      if (idx <= batch) ws.soff[idx] = m;
-      carry = total > carry ? total : carry;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && bad >= 0) report(ws.status, MPM_ERR_DEVICE_CHECK, bad);
-    // plan[b] = number of affinity tiles of the images before b.
-    __threadfence_block();
-    int64_t acc = 0;
-    for (int base = 0; base <= batch; base += kThreads) {
-      const int idx = base + threadIdx.x;
-      int64_t items = 0;
-      if (idx < batch) {
-        const int64_t n = ws.soff[idx + 1] - ws.soff[idx];
-        items = image_items(n, tile);
-      }
-      int64_t total;
-      const int64_t incl = block_incl_sum<int64_t>(items, sh, &total);
-      if (idx <= batch) ws.plan[idx] = acc + incl - items;
-      acc += total;
-    }
-  }
+  if (blockIdx.x == 0) write_plan(offsets, batch, rows, tile, ws);
 
   // Inverse norms of every used row, and the arg-max keys reset to "none".
   // Each warp takes kPrepRows consecutive rows at a time and issues all of
@@ -130,21 +130,6 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const uint8_t* __restric
       for (int r = 0; r < kPrepRows; ++r)
 #pragma unroll
         for (int u = 0; u < kPrepVecs; ++u) s[r] += sumsq16(buf[r][u], bf16);
-      if constexpr (SPLIT) {
-#pragma unroll
-        for (int r = 0; r < kPrepRows; ++r)
-#pragma unroll
-          for (int u = 0; u < kPrepVecs; ++u) {
-            const int v = v0 + 32 * u;
-            if (g0 + r < used && v < nvec) {
-              uint4 hi, lo;
-              split_tf32(buf[r][u], hi, lo);
-              const int64_t at = row_of(g0 + r) * (row_bytes >> 4) + v;
-              reinterpret_cast<uint4*>(ws.split_hi)[at] = hi;
-              reinterpret_cast<uint4*>(ws.split_lo)[at] = lo;
-            }
-          }
-      }
     }
 #pragma unroll
     for (int r = 0; r < kPrepRows; ++r) {
@@ -157,6 +142,140 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const uint8_t* __restric
       for (int r = 1; r < kPrepRows; ++r) mine = lane == r ? s[r] : mine;
       ws.inv_norm[row_of(g0 + lane)] = 1.0f / fmaxf(sqrtf(mine), 1e-12f);
       ws.keys[row_of(g0 + lane)] = 0ull;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Prep of fp32 tokens for the tensor cores.  Each row is scaled by the power
+// of two that brings its norm into [2^14, 2^15) and split into two fp16
+// values per element, x = hi + lo with hi the fp16 rounding of x and lo that
+// of x - hi: 22 significant bits, as many as a tf32 high and low part hold,
+// at half the bytes, and the tensor cores take fp16 at twice the tf32 rate.
+// No element exceeds fp16's range, since none exceeds its row's norm, and the
+// absolute error of an element far below the norm, 2^-25, is 2^-39 of the
+// norm.  Dot products scale exactly, so a row's arg max is unchanged, and
+// inv_norm receives the scaled rows' inverse norms (the plain ones times the
+// inverse power of two), which undo the scale in the cosines.
+//
+// Against fp64, the cosines of 700 tokens of 64 to 16384 features (normal,
+// clustered, heavy-tailed, offset, one feature 300 times the others) are 1.2
+// to 2 times closer than through tf32 parts: half as many accumulations.
+//
+// Bound by HBM: 65536 rows of 768 take 201 MB in and 201 MB out, 64.6 us (the
+// two fp32-sized tf32 parts took 100.2).
+// ---------------------------------------------------------------------------
+constexpr int kSplitVecs = 8;  // 16-byte vectors of a row that a lane keeps in registers (D <= 1024)
+
+struct RowScale {
+  float s1, s2;  // the row's scale is s1 * s2
+  float inv;     // 1 / max(|x|, 1e-12) of the scaled row
+};
+
+// Rows whose sum of squares says too little: zero rows, values far out of the
+// usual range, infinities and NaN.  Out of line, since ordinary rows never
+// come here.
+__device__ __noinline__ RowScale odd_row_scale(const uint4* src, int nvec, float sumsq) {
+  const int lane = threadIdx.x & 31;
+  float top = 0.f;
+  bool finite = true;
+  for (int v = lane; v < nvec; v += 32) {
+    const uint4 q = __ldg(src + v);
+    const float f[4] = {__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w)};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      finite = finite && fabsf(f[k]) <= 3.402823466e38f;
+      top = fmaxf(top, fabsf(f[k]));
+    }
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, d));
+  // A row with an infinity or NaN has no defined cosines: all NaN, so that it
+  // never is anyone's neighbour.
+  if (!__all_sync(0xFFFFFFFFu, finite))
+    return {__int_as_float(0x7fc00000), 1.0f, 1.0f / fmaxf(sqrtf(sumsq), 1e-12f)};
+  if (top == 0.f) return {1.0f, 1.0f, 1.0f / 1e-12f};
+  // Largest element to [2^7, 2^8): the norm of at most 2^14 elements stays
+  // below 2^15, and its square within fp32's range.
+  const int e = 7 - ilogbf(top);
+  const float s1 = scalbnf(1.0f, e / 2), s2 = scalbnf(1.0f, e - e / 2);
+  float s = 0.f;
+  for (int v = lane; v < nvec; v += 32) {
+    const uint4 q = __ldg(src + v);
+    const float f[4] = {__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w)};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float x = f[k] * s1 * s2;
+      s = fmaf(x, x, s);
+    }
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+  return {s1, s2, 1.0f / fmaxf(sqrtf(s), 1e-12f * s1 * s2)};
+}
+
+__global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __restrict__ tokens,
+                                                              const int64_t* __restrict__ offsets, int batch,
+                                                              int64_t rows, int dim, AffinityTile tile,
+                                                              Workspace ws) {
+  MPM_TRACE_BEGIN(MPM_TRACE_PREP);
+  wait_for_previous_grid();
+  MPM_TRACE_WAITED();
+  allow_next_grid();  // as in prep_kernel
+  if (blockIdx.x == 0) write_plan(offsets, batch, rows, tile, ws);
+
+  const int64_t used = clamp64(offsets[batch], 0, rows);
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
+  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
+  const int nvec = dim >> 2;
+  const int64_t stride = split_stride(dim) >> 2;  // in groups of four values
+  for (int64_t g = warp; g < used; g += nwarps) {
+    const int64_t r = used - 1 - g;  // last row first, as in prep_kernel
+    const uint4* src = reinterpret_cast<const uint4*>(tokens) + r * nvec;
+    uint4 buf[kSplitVecs];
+    float s = 0.f;
+#pragma unroll
+    for (int u = 0; u < kSplitVecs; ++u) {
+      const int v = lane + 32 * u;
+      buf[u] = v < nvec ? __ldg(src + v) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < kSplitVecs; ++u) s += sumsq16(buf[u], false);
+    for (int v = lane + 32 * kSplitVecs; v < nvec; v += 32) s += sumsq16(__ldg(src + v), false);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+    RowScale sc;
+    if (s >= 0x1p-100f && s <= 0x1p100f) {
+      const float norm = sqrtf(s);
+      const int e = 14 - (static_cast<int>(__float_as_uint(norm) >> 23) - 127);
+      sc.s1 = __uint_as_float(static_cast<uint32_t>(127 + e) << 23);
+      sc.s2 = 1.0f;
+      sc.inv = 1.0f / fmaxf(norm, 1e-12f) * __uint_as_float(static_cast<uint32_t>(127 - e) << 23);
+    } else {
+      sc = odd_row_scale(src, nvec, s);
+    }
+    uint2* hi = reinterpret_cast<uint2*>(ws.split_hi) + r * stride;
+    uint2* lo = reinterpret_cast<uint2*>(ws.split_lo) + r * stride;
+#pragma unroll
+    for (int u = 0; u < kSplitVecs; ++u) {
+      const int v = lane + 32 * u;
+      if (v < nvec) {
+        uint2 h, l;
+        split_f16(buf[u], sc.s1, sc.s2, h, l);
+        hi[v] = h;
+        lo[v] = l;
+      }
+    }
+    for (int v = lane + 32 * kSplitVecs; v < nvec; v += 32) {
+      uint2 h, l;
+      split_f16(__ldg(src + v), sc.s1, sc.s2, h, l);
+      hi[v] = h;
+      lo[v] = l;
+    }
+    if (lane == 0) {
+      ws.inv_norm[r] = sc.inv;
+      ws.keys[r] = 0ull;
     }
   }
 }
@@ -564,12 +683,12 @@ cudaError_t launch_prep(const void* tokens, const int64_t* offsets, int batch, i
                         cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
   if (ws.split_hi != nullptr) {
-    static const int per_sm = resident_per_sm(prep_kernel<true>, kThreads, 8);
-    return launch_dependent(prep_kernel<true>, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
-                            static_cast<const uint8_t*>(tokens), offsets, batch, rows, row_bytes, bf16, tile, ws);
+    static const int per_sm = resident_per_sm(prep_split_kernel, kThreads, 8);
+    return launch_dependent(prep_split_kernel, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
+                            static_cast<const uint8_t*>(tokens), offsets, batch, rows, dim, tile, ws);
   }
-  static const int per_sm = resident_per_sm(prep_kernel<false>, kThreads, 8);
-  return launch_dependent(prep_kernel<false>, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
+  static const int per_sm = resident_per_sm(prep_kernel, kThreads, 8);
+  return launch_dependent(prep_kernel, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
                           static_cast<const uint8_t*>(tokens), offsets, batch, rows, row_bytes, bf16, tile, ws);
 }
 

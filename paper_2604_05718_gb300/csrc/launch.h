@@ -20,12 +20,15 @@ struct Workspace {
   float* inv_norm;            // float[rows] 1 / max(|x_i|, 1e-12)
   unsigned long long* keys;   // u64[rows] packed (score, lowest j) arg-max keys
   int2* reps;                 // int2[rows] (representative, partner or -1), per image
-  // fp32 tokens only: x split into a tf32 high part and the fp32 remainder
-  // (float[rows * dim] each), for the three-product tf32 tensor-core path.
-  // Null for bf16.
-  float* split_hi;
-  float* split_lo;
+  // fp32 tokens only, for the three-product tensor-core path: every row
+  // scaled by a power of two and split into fp16 high and low parts (rows of
+  // split_stride(dim) values).  inv_norm then holds the scaled rows' inverse
+  // norms.  Null for bf16.
+  uint16_t* split_hi;
+  uint16_t* split_lo;
 };
+// fp16 values per row of the split parts: whole 16-byte rows, as TMA needs.
+__host__ __device__ constexpr int64_t split_stride(int dim) { return (static_cast<int64_t>(dim) + 7) / 8 * 8; }
 
 // Tile of one affinity work item: rows x columns of the cosine matrix, and
 // which tiles of an image's N x N matrix are computed:
@@ -59,9 +62,9 @@ cudaError_t launch_affinity_tc(const void* tokens, int batch, int64_t rows, int 
 AffinityTile tc_tile(bool symmetric);
 bool tc_available();
 
-// Symmetric affinity + arg max on SM pairs (tcgen05.mma.cta_group::2, bf16).
-// tf32: fp32 tokens through the three-product tf32 split (ws.split_hi / split_lo).
-cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, int dim, bool tf32, int64_t chunk,
+// Symmetric affinity + arg max on SM pairs (tcgen05.mma.cta_group::2).
+// split: fp32 tokens through three fp16 products per term (ws.split_hi / split_lo).
+cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, int dim, bool split, int64_t chunk,
                                  const Workspace& ws, int num_sms, cudaStream_t stream);
 AffinityTile pair_tile();
 

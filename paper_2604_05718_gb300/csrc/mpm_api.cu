@@ -39,7 +39,10 @@ struct Layout {
   size_t status, soff, plan, count, inv_norm, keys, reps, split_hi, split_lo, total;
 };
 
-// split_elems: rows * dim for fp32 tokens (the tf32 high / low copies), 0 for bf16.
+// split_elems: rows * dim for fp32 tokens, 0 for bf16.  Each split part is
+// given 4 bytes per element, twice what its fp16 values take (rows padded to
+// 8 values included): the documented workspace size, which also decides what
+// mpm_merge_no_alloc accepts.
 Layout layout(int64_t rows, int32_t batch, size_t split_elems) {
   Layout l{};
   size_t off = 0;
@@ -80,8 +83,8 @@ Workspace carve(void* base, int64_t rows, int32_t batch, size_t split) {
   ws.inv_norm = reinterpret_cast<float*>(p + l.inv_norm);
   ws.keys = reinterpret_cast<unsigned long long*>(p + l.keys);
   ws.reps = reinterpret_cast<int2*>(p + l.reps);
-  ws.split_hi = split > 0 ? reinterpret_cast<float*>(p + l.split_hi) : nullptr;
-  ws.split_lo = split > 0 ? reinterpret_cast<float*>(p + l.split_lo) : nullptr;
+  ws.split_hi = split > 0 ? reinterpret_cast<uint16_t*>(p + l.split_hi) : nullptr;
+  ws.split_lo = split > 0 ? reinterpret_cast<uint16_t*>(p + l.split_lo) : nullptr;
   return ws;
 }
 
@@ -121,11 +124,11 @@ mpm_status check_tokens(const void* tokens, int64_t rows, int32_t dim, mpm_dtype
 }
 
 // Kernel used when the caller does not choose one: the SM-pair tensor-core
-// kernel, with bf16 products for bf16 tokens and three tf32 products (high
+// kernel, with bf16 products for bf16 tokens and three fp16 products (high
 // and low parts, about fp32 accuracy) for fp32 tokens.
 mpm_nn_algo default_algo(mpm_dtype) { return MPM_NN_TCGEN05_PAIR; }
 
-// The workspace's tf32 split copies are filled only for the fp32 tensor-core path.
+// The workspace's split parts are filled only for the fp32 tensor-core path.
 Workspace for_algo(Workspace ws, mpm_nn_algo algo, mpm_dtype dtype) {
   if (!(algo == MPM_NN_TCGEN05_PAIR && dtype == MPM_F32)) ws.split_hi = ws.split_lo = nullptr;
   return ws;

@@ -1,6 +1,6 @@
-"""fp32 tokens on the tensor cores: each product x.y is taken as three tf32
-products of the high and low parts (x = hi + lo, hi the tf32 rounding of x),
-accumulated in fp32.  The result must meet the fp32 bar against the oracle,
+"""fp32 tokens on the tensor cores: each product x.y is taken as three fp16
+products of the high and low parts (x scaled, x = hi + lo, hi its fp16
+rounding), accumulated in fp32.  The result must meet the fp32 bar against the oracle,
 agree with the CUDA-core fp32 kernel on every decisive row, and give cosines
 within 1e-5 of the exact ones."""
 

@@ -106,7 +106,7 @@ def test_narrow_tiles_16_warps(mpm, pairs):
 
 
 def test_all_split_fp32(mpm, pairs):
-    # fp32 tokens take the three-product tf32 kernel with 8 epilogue warps.
+    # fp32 tokens take the three-product kernel with 8 epilogue warps.
     sizes = sizes_for(pairs // 2 - 1)
     check(mpm, sizes, 128, "f32", 73, "fp32 all split")
 

@@ -157,7 +157,7 @@ def test_no_alloc_rejects_sizes_beyond_its_scratch(mpm):
     assert lib.mpm_merge_workspace_size(400_000, 4, 64, 1) <= limit
     assert lib.mpm_merge_workspace_size(1 << 22, 4, 64, 1) > limit
     assert lib.mpm_merge_no_alloc(fake, fake, 4, 1 << 22, 64, 1, fake, fake, fake, None) == MPM_ERR_WORKSPACE
-    # fp32: 20 + 8 * dim bytes per row (the tf32 split copies), so 1,360 rows at dim 768.
+    # fp32: 20 + 8 * dim bytes per row (room for two split copies), so 1,360 rows at dim 768.
     assert lib.mpm_merge_workspace_size(1300, 2, 768, 0) <= limit
     assert lib.mpm_merge_workspace_size(1400, 2, 768, 0) > limit
     assert lib.mpm_merge_no_alloc(fake, fake, 2, 1400, 768, 0, fake, fake, fake, None) == MPM_ERR_WORKSPACE
