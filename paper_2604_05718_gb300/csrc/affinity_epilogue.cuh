@@ -75,50 +75,80 @@ __device__ __forceinline__ void mul_f32x2(float& r0, float& r1, float a0, float 
       : "=f"(r0), "=f"(r1)
       : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
 }
-// One 16-column piece of a warp's slice: row candidates into two running
-// maxima (even and odd columns), and, with COL, the column maxima and their
-// winning rows of these 16 columns into the per-warp scratch entries
-// slot .. slot + 15.  Columns go in pairs, two products to an instruction and
-// two results to a 16-byte store: the epilogue's issue slots and shared-memory
-// accesses are taken from the tensor cores' (one store per column and single
-// products: vit_b step 202.9 instead of 201.7 us with paired stores and 200.9
-// with both; mixed 237.1, 234.8 and 231.6).
-template <bool DIAG, bool COL>
-__device__ __forceinline__ void epilogue_piece(const uint32_t (&v)[16], const float* sc, int c, int jd, float& best0,
-                                               int& bj0, float& best1, int& bj1, float inv_i, int lane,
-                                               uint2* scratch, int slot) {
+
+// Running row maximum over groups of eight columns: the best score, the first
+// column of the group it came from, and that group's first seven scores, from
+// which the column is found once at the end.  (An index per column took three
+// instructions a column, groups of four take 2, of eight 1.75: vit_b step
+// 202.2, 200.6 and 200.3 us, mixed 233.8, 229.4 and 228.9.)
+struct RowBest {
+  float top = -INFINITY;
+  float s[7] = {};
+  int at = -1;
+
+  // Scores of columns c .. c + 7.  A group replaces the best only when it is
+  // larger, so the lowest column wins ties; NaN scores never win.
+  __device__ __forceinline__ void take(const float (&x)[8], int c) {
+    float m;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(x[0]), "f"(x[1]), "f"(x[2]));
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(m), "f"(x[3]), "f"(x[4]));
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(m), "f"(x[5]), "f"(x[6]));
+    m = fmaxf(m, x[7]);
+    if (m > top) {
+      top = m;
+      at = c;
 #pragma unroll
-  for (int k = 0; k < 16; k += 4) {
-    const float4 s4 = *reinterpret_cast<const float4*>(sc + c + k);
-    float sv[4];
-    mul_f32x2(sv[0], sv[1], __uint_as_float(v[k]), __uint_as_float(v[k + 1]), s4.x, s4.y);
-    mul_f32x2(sv[2], sv[3], __uint_as_float(v[k + 2]), __uint_as_float(v[k + 3]), s4.z, s4.w);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float s = sv[u];
-      const int j = c + k + u;
-      if (u & 1) {
-        if (s > best1 && (!DIAG || j != jd)) {
-          best1 = s;
-          bj1 = j;
-        }
-      } else {
-        if (s > best0 && (!DIAG || j != jd)) {
-          best0 = s;
-          bj0 = j;
-        }
-      }
+      for (int i = 0; i < 7; ++i) s[i] = x[i];
     }
   }
+  // The column of the best score (-1 when there is none).
+  __device__ __forceinline__ int column() const {
+    int i = 7;
+#pragma unroll
+    for (int k = 6; k >= 0; --k)
+      if (s[k] == top) i = k;
+    return at < 0 ? -1 : at + i;
+  }
+};
+
+// One 16-column piece of a warp's slice: row candidates into the running row
+// maximum, and, with COL, the column maxima and their winning rows of these
+// 16 columns into the per-warp scratch entries slot .. slot + 15.  Columns go
+// in pairs, two products to an instruction and two results to a 16-byte
+// store: the epilogue's issue slots and shared-memory accesses are taken from
+// the tensor cores' (one store per column and single products: vit_b step
+// 202.9 instead of 201.7 us with paired stores and 200.9 with both; mixed
+// 237.1, 234.8 and 231.6).
+template <bool DIAG, bool COL>
+__device__ __forceinline__ void epilogue_piece(const uint32_t (&v)[16], const float* sc, int c, int jd, RowBest& best,
+                                               float inv_i, uint2* scratch, int slot, bool writer) {
+#pragma unroll
+  for (int k = 0; k < 16; k += 8) {
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; u += 4) {
+      const float4 s4 = *reinterpret_cast<const float4*>(sc + c + k + u);
+      mul_f32x2(x[u], x[u + 1], __uint_as_float(v[k + u]), __uint_as_float(v[k + u + 1]), s4.x, s4.y);
+      mul_f32x2(x[u + 2], x[u + 3], __uint_as_float(v[k + u + 2]), __uint_as_float(v[k + u + 3]), s4.z, s4.w);
+    }
+    if (DIAG) {
+      // A token is no candidate of its own.  (Masking only the 32 columns that
+      // hold the warp's diagonal, behind a uniform branch, was 3% slower.)
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (c + k + u == jd) x[u] = -INFINITY;
+    }
+    best.take(x, c + k);
+  }
   if (COL) {
-    const bool writer = lane == 0;
 #pragma unroll
     for (int k = 0; k < 16; k += 2) {
       float s0, s1;
       mul_f32x2(s0, s1, __uint_as_float(v[k]), __uint_as_float(v[k + 1]), inv_i, inv_i);
       const float m0 = warp_max_f32(s0), m1 = warp_max_f32(s1);
       const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, s0 == m0), b1 = __ballot_sync(0xFFFFFFFFu, s1 == m1);
-      if (writer) *reinterpret_cast<uint4*>(scratch + slot + k) = make_uint4(__float_as_uint(m0), b0, __float_as_uint(m1), b1);
+      if (writer)
+        *reinterpret_cast<uint4*>(scratch + slot + k) = make_uint4(__float_as_uint(m0), b0, __float_as_uint(m1), b1);
     }
   }
 }
@@ -138,18 +168,17 @@ __device__ __forceinline__ unsigned long long column_candidate(const uint2* scra
 // A warp's whole COLS-column slice of one accumulator (TMEM columns
 // taddr .. taddr + COLS - 1, tile columns c0 ..), read in 16-column pieces
 // with the next piece's load in flight while the current one is processed.
-// The loop body covers two pieces (32 columns).  Row candidates use two independent running maxima (even and odd columns),
-// merged at the end with the lowest-index rule, to halve the dependent
-// chain.  colcand[h] receives the column candidate of tile column
-// c0 + 32 h + lane (0 when none).
+// The loop body covers two pieces (32 columns).  DIAG: the slice may hold the
+// row's own column, jd.  colcand[h] receives the column candidate of tile
+// column c0 + 32 h + lane (0 when none).
 template <int COLS, bool DIAG, bool COL>
 __device__ __forceinline__ void epilogue_slice(uint32_t taddr, const float* sc, int c0, int jd, float& best,
                                                int& bj, float inv_i, int lane, int row_base, int n, int col0,
                                                int origin, uint2* scratch,
                                                unsigned long long (&colcand)[COLS / 32]) {
   static_assert(COLS % 32 == 0, "slices are whole 32-column pairs of pieces");
-  float best0 = -INFINITY, best1 = -INFINITY;
-  int bj0 = -1, bj1 = -1;
+  const bool writer = lane == 0;
+  RowBest rows;
   uint32_t va[16], vb[16];
   ptx::tmem_ld_32x32b_x16(taddr, va);
   ptx::tmem_wait_ld(va);
@@ -157,10 +186,10 @@ __device__ __forceinline__ void epilogue_slice(uint32_t taddr, const float* sc, 
   for (int h = 0; h < COLS / 32; ++h) {
     const int c = c0 + 32 * h;
     ptx::tmem_ld_32x32b_x16(taddr + 32 * h + 16, vb);
-    epilogue_piece<DIAG, COL>(va, sc, c, jd, best0, bj0, best1, bj1, inv_i, lane, scratch, 0);
+    epilogue_piece<DIAG, COL>(va, sc, c, jd, rows, inv_i, scratch, 0, writer);
     ptx::tmem_wait_ld(vb);
     if (h + 1 < COLS / 32) ptx::tmem_ld_32x32b_x16(taddr + 32 * h + 32, va);
-    epilogue_piece<DIAG, COL>(vb, sc, c + 16, jd, best0, bj0, best1, bj1, inv_i, lane, scratch, 16);
+    epilogue_piece<DIAG, COL>(vb, sc, c + 16, jd, rows, inv_i, scratch, 16, writer);
     if (COL) {
       const unsigned long long key = column_candidate(scratch, lane, row_base, n, col0 + c + lane, origin);
 #pragma unroll
@@ -169,31 +198,25 @@ __device__ __forceinline__ void epilogue_slice(uint32_t taddr, const float* sc, 
     }
     if (h + 1 < COLS / 32) ptx::tmem_wait_ld(va);
   }
-  // Merge the two chains: larger score, lower column on equal scores.
-  if (best1 > best0 || (best1 == best0 && bj1 >= 0 && (bj0 < 0 || bj1 < bj0))) {
-    best0 = best1;
-    bj0 = bj1;
-  }
-  if (bj0 >= 0 && (bj < 0 || best0 > best || (best0 == best && bj0 < bj))) {
-    best = best0;
-    bj = bj0;
-  }
+  best = rows.top;
+  bj = rows.column();
 }
 
 // The same slice with the 32-column loop left rolled (`steps` steps of 32
 // columns), for 128-column slices, whose unrolled code is twice as long:
 // the column candidate of tile column c0 + 32 h + lane goes straight to
 // colkeys[32 h] (colkeys points at this lane's first column) instead of a
-// register array, which would need the loop unrolled.  (Measured on vit_b: step 0.2051-0.2054
-// against 0.2069-0.2073 ms unrolled; the 64-column slices of the 16-warp
-// epilogue stay unrolled, where the rolled loop was 1.4% slower.)
+// register array, which would need the loop unrolled.  (Measured on vit_b:
+// step 0.2051-0.2054 against 0.2069-0.2073 ms unrolled; the 64-column slices
+// of the 16-warp epilogue stay unrolled, where the rolled loop was 1.4%
+// slower.)
 template <bool DIAG, bool COL>
 __device__ __forceinline__ void epilogue_slice_rolled(uint32_t taddr, const float* sc, int c0, int jd, float& best,
                                                       int& bj, float inv_i, int lane, int row_base, int n,
                                                       int col0, int origin, uint2* scratch,
                                                       unsigned long long* colkeys, int steps) {
-  float best0 = -INFINITY, best1 = -INFINITY;
-  int bj0 = -1, bj1 = -1;
+  const bool writer = lane == 0;
+  RowBest rows;
   uint32_t va[16], vb[16];
   ptx::tmem_ld_32x32b_x16(taddr, va);
   ptx::tmem_wait_ld(va);
@@ -201,25 +224,19 @@ __device__ __forceinline__ void epilogue_slice_rolled(uint32_t taddr, const floa
   for (int h = 0; h < steps; ++h) {
     const int c = c0 + 32 * h;
     ptx::tmem_ld_32x32b_x16(taddr + 32 * h + 16, vb);
-    epilogue_piece<DIAG, COL>(va, sc, c, jd, best0, bj0, best1, bj1, inv_i, lane, scratch, 0);
+    epilogue_piece<DIAG, COL>(va, sc, c, jd, rows, inv_i, scratch, 0, writer);
     ptx::tmem_wait_ld(vb);
     const bool more = h + 1 < steps;
     if (more) ptx::tmem_ld_32x32b_x16(taddr + 32 * h + 32, va);
-    epilogue_piece<DIAG, COL>(vb, sc, c + 16, jd, best0, bj0, best1, bj1, inv_i, lane, scratch, 16);
+    epilogue_piece<DIAG, COL>(vb, sc, c + 16, jd, rows, inv_i, scratch, 16, writer);
     if (COL) {
       const unsigned long long key = column_candidate(scratch, lane, row_base, n, col0 + c + lane, origin);
       if (key != 0ull) atomicMax(colkeys + 32 * h, key);
     }
     if (more) ptx::tmem_wait_ld(va);
   }
-  if (best1 > best0 || (best1 == best0 && bj1 >= 0 && (bj0 < 0 || bj1 < bj0))) {
-    best0 = best1;
-    bj0 = bj1;
-  }
-  if (bj0 >= 0 && (bj < 0 || best0 > best || (best0 == best && bj0 < bj))) {
-    best = best0;
-    bj = bj0;
-  }
+  best = rows.top;
+  bj = rows.column();
 }
 
 }  // namespace mpm
