@@ -129,7 +129,9 @@ __device__ __forceinline__ int find_item_image(const int64_t* __restrict__ plan,
 // has C - (I >> 1) of them; row blocks 2m and 2m+1 have 2(C - m) together.
 // Upper square (rows == cols): the R (R + 1) / 2 tiles with J >= I.
 __host__ __device__ __forceinline__ int64_t affinity_tiles(int64_t n, int rows, int cols, int mode) {
-  const int64_t r = (n + rows - 1) / rows, c = (n + cols - 1) / cols;
+  // n < 2^31: 32-bit quotients (64-bit ones are long subroutines).
+  const uint32_t un = static_cast<uint32_t>(n), ur = static_cast<uint32_t>(rows), uc = static_cast<uint32_t>(cols);
+  const int64_t r = (un + ur - 1) / ur, c = (un + uc - 1) / uc;
   if (mode == AffinityTile::kDense) return r * c;
   if (mode == AffinityTile::kUpperSquare) return r * (r + 1) / 2;
   const int64_t q = r / 2;
@@ -140,7 +142,7 @@ __host__ __device__ __forceinline__ int64_t affinity_tiles(int64_t n, int rows, 
 // image when t.chunk == 0; the last chunk may be shorter).
 __host__ __device__ __forceinline__ int64_t image_items(int64_t n, const AffinityTile& t) {
   if (t.chunk <= 0 || n <= t.chunk) return affinity_tiles(n, t.rows, t.cols, t.mode);
-  const int64_t full = n / t.chunk, last = n - full * t.chunk;
+  const int64_t full = static_cast<uint32_t>(n) / static_cast<uint32_t>(t.chunk), last = n - full * t.chunk;
   return full * affinity_tiles(t.chunk, t.rows, t.cols, t.mode) +
          (last > 0 ? affinity_tiles(last, t.rows, t.cols, t.mode) : 0);
 }
@@ -153,8 +155,8 @@ struct ChunkItem {
 __device__ __forceinline__ ChunkItem locate_chunk(int64_t local, int64_t n, const AffinityTile& t) {
   if (t.chunk <= 0 || n <= t.chunk) return {0, n, local};
   const int64_t per = affinity_tiles(t.chunk, t.rows, t.cols, t.mode);
-  const int64_t full = n / t.chunk;
-  const int64_t c = local / per;
+  const int64_t full = static_cast<uint32_t>(n) / static_cast<uint32_t>(t.chunk);
+  const int64_t c = ((local | per) >> 32) == 0 ? static_cast<uint32_t>(local) / static_cast<uint32_t>(per) : local / per;
   if (c < full) return {c * t.chunk, t.chunk, local - c * per};
   return {full * t.chunk, n - full * t.chunk, local - full * per};
 }

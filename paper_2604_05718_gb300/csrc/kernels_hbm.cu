@@ -12,8 +12,6 @@ namespace mpm {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kPrepRows = 2;   // rows per warp iteration in prep_kernel
-constexpr int kPrepVecs = 3;   // 16-byte vectors per lane and row per pass (one pass at D = 768 bf16)
 
 __device__ __forceinline__ int64_t clamp64(int64_t v, int64_t lo, int64_t hi) {
   return v < lo ? lo : (v > hi ? hi : v);
@@ -34,61 +32,81 @@ struct ImageCursor {
 
 // ---------------------------------------------------------------------------
 // Prep: status reset, offsets sanitisation + work plan (block 0), inverse
-// row norms and key reset (all blocks).
+// row norms and key reset (all other blocks).  Large batches are bound by
+// HBM; small ones by the dependent loads of block 0, whose plan takes one
+// pass through shared memory and no rows of its own (430 rows in 3 images: 3.0
+// -> 1.3 us).
 // ---------------------------------------------------------------------------
+// Sanitised offsets and work plan, by one block:
+//   soff[b] = min(rows, max_{b' <= b} max(off[b'], 0)), non-decreasing and in
+//             range whatever the caller passed (violations are reported);
+//   plan[b] = number of affinity tiles of the images before b.
 __device__ __forceinline__ void write_plan(const int64_t* __restrict__ offsets, int batch, int64_t rows,
                                            const AffinityTile& tile, const Workspace& ws) {
   __shared__ int64_t sh[32];
+  __shared__ int64_t ends[kThreads + 1];
   __shared__ int bad;
+  int64_t off0 = 0;
   if (threadIdx.x == 0) {
     ws.status[0] = 0;
     ws.status[1] = 0;
     ws.status[2] = 0;
-    bad = -1;
+    off0 = offsets[0];
+    bad = off0 != 0 ? 0 : -1;
+    ends[0] = clamp64(off0, 0, rows);
+    ws.soff[0] = ends[0];
   }
   __syncthreads();
-  // soff[b] = min(rows, max_{b' <= b} max(off[b'], 0)): non-decreasing and
-  // in range whatever the caller passed; violations are reported.
-  int64_t carry = 0;
-  for (int base = 0; base <= batch; base += kThreads) {
-    const int idx = base + threadIdx.x;
-    int64_t raw = 0, prev = 0;
-    if (idx <= batch) {
-      raw = offsets[idx];
-      prev = idx > 0 ? offsets[idx - 1] : 0;
-      if ((idx == 0 && raw != 0) || raw < prev || raw > rows) atomicCAS(&bad, -1, idx);
-    }
-    int64_t v = idx <= batch ? clamp64(raw, 0, rows) : 0;
-    int64_t total;
-    int64_t m = block_incl_max<int64_t>(v, sh, &total, 0);
-    m = m > carry ? m : carry;
-    if (idx <= batch) ws.soff[idx] = m;
-    carry = total > carry ? total : carry;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0 && bad >= 0) report(ws.status, MPM_ERR_DEVICE_CHECK, bad);
-  // plan[b] = number of affinity tiles of the images before b.
-  __threadfence_block();
   int64_t acc = 0;
-  for (int base = 0; base <= batch; base += kThreads) {
+  for (int base = 0; base < batch; base += kThreads) {
+    // Image `idx`: from soff[idx], which the thread before has, to soff[idx + 1].
     const int idx = base + threadIdx.x;
+    int64_t end = 0;
+    if (idx < batch) {
+      const int64_t raw = offsets[idx + 1];
+      if (raw < offsets[idx] || raw > rows) atomicCAS(&bad, -1, idx + 1);
+      end = clamp64(raw, 0, rows);
+    }
+    const int64_t carry = ends[0];
+    int64_t last;
+    end = block_incl_max<int64_t>(end, sh, &last, 0);
+    end = end > carry ? end : carry;
+    ends[threadIdx.x + 1] = end;
+    __syncthreads();
     int64_t items = 0;
     if (idx < batch) {
-      const int64_t n = ws.soff[idx + 1] - ws.soff[idx];
-      items = image_items(n, tile);
+      ws.soff[idx + 1] = end;
+      items = image_items(end - ends[threadIdx.x], tile);
     }
     int64_t total;
     const int64_t incl = block_incl_sum<int64_t>(items, sh, &total);
-    if (idx <= batch) ws.plan[idx] = acc + incl - items;
+    if (idx < batch) ws.plan[idx] = acc + incl - items;
     acc += total;
+    if (threadIdx.x == 0) ends[0] = last > carry ? last : carry;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    ws.plan[batch] = acc;
+    if (bad >= 0) report(ws.status, MPM_ERR_DEVICE_CHECK, bad);
   }
 }
 
+// This warp's number among the warps of `blocks` blocks, this one being
+// `block`.  Few rows (spread) are dealt across the blocks, so that they use
+// every SM; a whole wave numbers a block's warps consecutively, so that its
+// rows lie together (dealt across, the pair average of 65536 x 768 bf16 took
+// 25.4 instead of 23.6 us).
+__device__ __forceinline__ int64_t warp_number(int block, int blocks, bool spread) {
+  const int w = static_cast<int>(threadIdx.x >> 5);
+  return spread ? static_cast<int64_t>(w) * blocks + block : static_cast<int64_t>(block) * (kThreads / 32) + w;
+}
+
+template <int ROWS, int VECS>
 __global__ void __launch_bounds__(kThreads) prep_kernel(const uint8_t* __restrict__ tokens,
                                                         const int64_t* __restrict__ offsets,
                                                         int batch, int64_t rows, int row_bytes,
                                                         bool bf16, AffinityTile tile,
-                                                        Workspace ws) {
+                                                        Workspace ws, bool spread) {
   MPM_TRACE_BEGIN(MPM_TRACE_PREP);
   wait_for_previous_grid();
   MPM_TRACE_WAITED();
@@ -97,49 +115,54 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const uint8_t* __restric
   // (The other kernels do not trigger early: blocks of a dependent grid
   // parked on SMs were measured to slow the bandwidth-bound kernels.)
   allow_next_grid();
-  if (blockIdx.x == 0) write_plan(offsets, batch, rows, tile, ws);
+  if (blockIdx.x == 0) {
+    write_plan(offsets, batch, rows, tile, ws);
+    return;
+  }
 
   // Inverse norms of every used row, and the arg-max keys reset to "none".
-  // Each warp takes kPrepRows consecutive rows at a time and issues all of
-  // their 16-byte loads before reducing, to keep enough bytes in flight.
+  // Each warp takes ROWS consecutive rows at a time and issues all of their
+  // 16-byte loads (VECS a lane and row; longer rows take more passes) before
+  // reducing, to keep enough bytes in flight.
   // The sweep runs from the last row to the first: the affinity kernel
   // starts with the first images, and those are then the ones this sweep
   // left in L2 (measured: 3.5 instead of 3.8 us per tile on vit_b).
   const int64_t used = clamp64(offsets[batch], 0, rows);
   auto row_of = [used](int64_t i) { return used - 1 - i; };
   const int lane = threadIdx.x & 31;
-  const int64_t warp = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
+  // The blocks after block 0 take the rows.
+  const int64_t warp = warp_number(blockIdx.x - 1, gridDim.x - 1, spread);
+  const int64_t nwarps = static_cast<int64_t>(gridDim.x - 1) * (kThreads / 32);
   const int nvec = row_bytes >> 4;
-  for (int64_t g0 = warp * kPrepRows; g0 < used; g0 += nwarps * kPrepRows) {
-    float s[kPrepRows];
+  for (int64_t g0 = warp * ROWS; g0 < used; g0 += nwarps * ROWS) {
+    float s[ROWS];
 #pragma unroll
-    for (int r = 0; r < kPrepRows; ++r) s[r] = 0.f;
-    for (int v0 = lane; v0 < nvec; v0 += 32 * kPrepVecs) {
-      uint4 buf[kPrepRows][kPrepVecs];
+    for (int r = 0; r < ROWS; ++r) s[r] = 0.f;
+    for (int v0 = lane; v0 < nvec; v0 += 32 * VECS) {
+      uint4 buf[ROWS][VECS];
 #pragma unroll
-      for (int r = 0; r < kPrepRows; ++r) {
+      for (int r = 0; r < ROWS; ++r) {
         const uint4* src = reinterpret_cast<const uint4*>(tokens + row_of(g0 + r) * row_bytes);
 #pragma unroll
-        for (int u = 0; u < kPrepVecs; ++u) {
+        for (int u = 0; u < VECS; ++u) {
           const int v = v0 + 32 * u;
           buf[r][u] = (g0 + r < used && v < nvec) ? __ldg(src + v) : make_uint4(0, 0, 0, 0);
         }
       }
 #pragma unroll
-      for (int r = 0; r < kPrepRows; ++r)
+      for (int r = 0; r < ROWS; ++r)
 #pragma unroll
-        for (int u = 0; u < kPrepVecs; ++u) s[r] += sumsq16(buf[r][u], bf16);
+        for (int u = 0; u < VECS; ++u) s[r] += sumsq16(buf[r][u], bf16);
     }
 #pragma unroll
-    for (int r = 0; r < kPrepRows; ++r) {
+    for (int r = 0; r < ROWS; ++r) {
 #pragma unroll
       for (int d = 16; d > 0; d >>= 1) s[r] += __shfl_xor_sync(0xFFFFFFFFu, s[r], d);
     }
-    if (lane < kPrepRows && g0 + lane < used) {
+    if (lane < ROWS && g0 + lane < used) {
       float mine = s[0];
 #pragma unroll
-      for (int r = 1; r < kPrepRows; ++r) mine = lane == r ? s[r] : mine;
+      for (int r = 1; r < ROWS; ++r) mine = lane == r ? s[r] : mine;
       ws.inv_norm[row_of(g0 + lane)] = 1.0f / fmaxf(sqrtf(mine), 1e-12f);
       ws.keys[row_of(g0 + lane)] = 0ull;
     }
@@ -217,17 +240,20 @@ __device__ __noinline__ RowScale odd_row_scale(const uint4* src, int nvec, float
 __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __restrict__ tokens,
                                                               const int64_t* __restrict__ offsets, int batch,
                                                               int64_t rows, int dim, AffinityTile tile,
-                                                              Workspace ws) {
+                                                              Workspace ws, bool spread) {
   MPM_TRACE_BEGIN(MPM_TRACE_PREP);
   wait_for_previous_grid();
   MPM_TRACE_WAITED();
   allow_next_grid();  // as in prep_kernel
-  if (blockIdx.x == 0) write_plan(offsets, batch, rows, tile, ws);
+  if (blockIdx.x == 0) {
+    write_plan(offsets, batch, rows, tile, ws);
+    return;
+  }
 
   const int64_t used = clamp64(offsets[batch], 0, rows);
   const int lane = threadIdx.x & 31;
-  const int64_t warp = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
+  const int64_t warp = warp_number(blockIdx.x - 1, gridDim.x - 1, spread);
+  const int64_t nwarps = static_cast<int64_t>(gridDim.x - 1) * (kThreads / 32);
   const int nvec = dim >> 2;
   const int64_t stride = split_stride(dim) >> 2;  // in groups of four values
   for (int64_t g = warp; g < used; g += nwarps) {
@@ -452,63 +478,57 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch,
 // ---------------------------------------------------------------------------
 // Pair average + compaction (Eq. 2): one warp per output row.
 // ---------------------------------------------------------------------------
-template <int R, int U>
+template <int U>
 __global__ void __launch_bounds__(kThreads) pair_average_kernel(const uint8_t* __restrict__ tokens,
                                                                 uint8_t* __restrict__ out,
                                                                 int batch, int64_t rows, int row_bytes,
                                                                 bool bf16, Workspace ws,
-                                                                const int64_t* __restrict__ out_offsets) {
+                                                                const int64_t* __restrict__ out_offsets,
+                                                                bool spread) {
   MPM_TRACE_BEGIN(MPM_TRACE_PAIR_AVERAGE);
   wait_for_previous_grid();
   MPM_TRACE_WAITED();
   const int lane = threadIdx.x & 31;
-  const int64_t warp = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
+  const int64_t warp = warp_number(blockIdx.x, gridDim.x, spread);
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
-  const int64_t total = clamp64(out_offsets[batch], 0, rows);
   const int nvec = row_bytes >> 4;
-  ImageCursor cur;
-  // Each warp writes R consecutive output rows per iteration; all loads of
-  // a pass are issued before any store.
-  for (int64_t t0 = warp * R; t0 < total; t0 += nwarps * R) {
-    const uint4* a[R];
-    const uint4* p[R];
-    uint4* dst[R];
-    bool live[R], pair[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int64_t t = t0 + r;
-      live[r] = t < total;
-      pair[r] = false;
-      a[r] = p[r] = nullptr;
-      dst[r] = reinterpret_cast<uint4*>(out + t * row_bytes);
-      if (live[r]) {
-        cur.locate(out_offsets, batch, t);
-        const int64_t in_base = ws.soff[cur.b];
-        const int2 rep = ws.reps[in_base + (t - cur.lo)];
-        pair[r] = rep.y >= 0;
-        a[r] = reinterpret_cast<const uint4*>(tokens + (in_base + rep.x) * row_bytes);
-        p[r] = reinterpret_cast<const uint4*>(tokens + (in_base + (pair[r] ? rep.y : rep.x)) * row_bytes);
-      }
+  int b = 0;
+  int64_t lo = 1, hi = 0, in_base = 0;  // empty: the first row is always looked up
+  int64_t total = INT64_MAX;  // known from the first look-up on
+  // A row's chain of dependent loads is what bounds few rows: the image
+  // search, its offsets, the pair, the tokens.  The total is loaded with the
+  // first image's offsets, not before them, and few rows spread over the SMs
+  // (1024 rows of 768 B: 3.6 -> 1.5 us).
+  for (int64_t t = warp; t < total; t += nwarps) {
+    if (t >= hi || t < lo) {
+      b = find_image(out_offsets, batch, t);
+      lo = __ldg(out_offsets + b);
+      hi = __ldg(out_offsets + b + 1);
+      in_base = ws.soff[b];
+      total = clamp64(__ldg(out_offsets + batch), 0, rows);
+      if (t >= total) break;
     }
+    const int2 rep = ws.reps[in_base + (t - lo)];
+    const bool pair = rep.y >= 0;
+    const uint4* a = reinterpret_cast<const uint4*>(tokens + (in_base + rep.x) * row_bytes);
+    const uint4* p = reinterpret_cast<const uint4*>(tokens + (in_base + (pair ? rep.y : rep.x)) * row_bytes);
+    uint4* dst = reinterpret_cast<uint4*>(out + t * row_bytes);
+    // All loads of a pass are issued before any store.
     for (int v0 = lane; v0 < nvec; v0 += 32 * U) {
-      uint4 va[R][U], vb[R][U];
+      uint4 va[U], vb[U];
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int v = v0 + 32 * u;
-          if (live[r] && v < nvec) {
-            va[r][u] = __ldcs(a[r] + v);
-            if (pair[r]) vb[r][u] = __ldcs(p[r] + v);
-          }
+      for (int u = 0; u < U; ++u) {
+        const int v = v0 + 32 * u;
+        if (v < nvec) {
+          va[u] = __ldcs(a + v);
+          if (pair) vb[u] = __ldcs(p + v);
         }
+      }
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int v = v0 + 32 * u;
-          if (live[r] && v < nvec) dst[r][v] = pair[r] ? avg16(va[r][u], vb[r][u], bf16) : va[r][u];
-        }
+      for (int u = 0; u < U; ++u) {
+        const int v = v0 + 32 * u;
+        if (v < nvec) dst[v] = pair ? avg16(va[u], vb[u], bf16) : va[u];
+      }
     }
   }
 }
@@ -658,6 +678,19 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const uint8_t* __restr
 
 int grid_for(int num_sms, int per_sm) { return (num_sms > 0 ? num_sms : 1) * per_sm; }
 
+// Blocks for `items` rows (or pairs of rows), one per warp and round: at most
+// one wave; fewer items get a block per four of them, spread over its warps'
+// numbers, so that no whole wave is launched for them.
+struct RowGrid {
+  int blocks;
+  bool spread;
+};
+RowGrid row_grid(int64_t items, int wave) {
+  const int64_t blocks = (items + 3) / 4;
+  if (blocks >= wave) return {wave, false};
+  return {blocks > 1 ? static_cast<int>(blocks) : 1, true};
+}
+
 // Blocks and rows per warp of the gather for `rows` grid rows: at most one
 // wave of blocks, and rows dealt evenly over its warps (at most kGatherRows a
 // warp and round).
@@ -684,12 +717,34 @@ cudaError_t launch_prep(const void* tokens, const int64_t* offsets, int batch, i
   const int row_bytes = dim * (bf16 ? 2 : 4);
   if (ws.split_hi != nullptr) {
     static const int per_sm = resident_per_sm(prep_split_kernel, kThreads, 8);
-    return launch_dependent(prep_split_kernel, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
-                            static_cast<const uint8_t*>(tokens), offsets, batch, rows, dim, tile, ws);
+    const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm) - 1);
+    return launch_dependent(prep_split_kernel, dim3(1 + g.blocks), dim3(kThreads), 0, stream,
+                            static_cast<const uint8_t*>(tokens), offsets, batch, rows, dim, tile, ws, g.spread);
   }
-  static const int per_sm = resident_per_sm(prep_kernel, kThreads, 8);
-  return launch_dependent(prep_kernel, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
-                          static_cast<const uint8_t*>(tokens), offsets, batch, rows, row_bytes, bf16, tile, ws);
+  // Rows and vectors per warp and round by the row's length, so that no load
+  // slot is empty: with 2 x 3 for every length, rows of 2 KiB took two passes
+  // (36864 of them 17.9 us, now 16.5) and rows of 768 B half the slots (32768
+  // of them 8.7, now 8.0); 4 x 3 and 1 x 3 were slower for 1.5 KiB.
+  const int nvec = row_bytes >> 4;
+  const auto launch = [&](auto kernel, int per_sm, int warp_rows) {
+    const RowGrid g = row_grid((rows + warp_rows - 1) / warp_rows, grid_for(num_sms, per_sm) - 1);
+    return launch_dependent(kernel, dim3(1 + g.blocks), dim3(kThreads), 0, stream, static_cast<const uint8_t*>(tokens),
+                            offsets, batch, rows, row_bytes, bf16, tile, ws, g.spread);
+  };
+  if (nvec <= 32) {
+    static const int per_sm = resident_per_sm(prep_kernel<4, 1>, kThreads, 8);
+    return launch(prep_kernel<4, 1>, per_sm, 4);
+  }
+  if (nvec <= 64) {
+    static const int per_sm = resident_per_sm(prep_kernel<3, 2>, kThreads, 8);
+    return launch(prep_kernel<3, 2>, per_sm, 3);
+  }
+  if (nvec <= 96) {
+    static const int per_sm = resident_per_sm(prep_kernel<2, 3>, kThreads, 8);
+    return launch(prep_kernel<2, 3>, per_sm, 2);
+  }
+  static const int per_sm = resident_per_sm(prep_kernel<2, 4>, kThreads, 8);
+  return launch(prep_kernel<2, 4>, per_sm, 2);
 }
 
 cudaError_t launch_mutual_compact(int batch, int64_t rows, int64_t chunk, const Workspace& ws, int32_t* out_map,
@@ -729,10 +784,11 @@ cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch,
                                 int dim, bool bf16, const Workspace& ws,
                                 const int64_t* out_offsets, int num_sms, cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
-  static const int per_sm = resident_per_sm(pair_average_kernel<1, 4>, kThreads, 8);
-  return launch_dependent(pair_average_kernel<1, 4>, dim3(grid_for(num_sms, per_sm)), dim3(kThreads), 0, stream,
+  static const int per_sm = resident_per_sm(pair_average_kernel<4>, kThreads, 8);
+  const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm));
+  return launch_dependent(pair_average_kernel<4>, dim3(g.blocks), dim3(kThreads), 0, stream,
                           static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch, rows,
-                          row_bytes, bf16, ws, out_offsets);
+                          row_bytes, bf16, ws, out_offsets, g.spread);
 }
 
 cudaError_t launch_decode_nn(int batch, int64_t rows, const Workspace& ws, int32_t* out_nn,
