@@ -728,14 +728,15 @@ cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, in
   void* hi = split ? static_cast<void*>(ws.split_hi) : const_cast<void*>(tokens);
   void* lo = split ? static_cast<void*>(ws.split_lo) : const_cast<void*>(tokens);
   if (hi == nullptr || lo == nullptr) return cudaErrorInvalidValue;
-  CUtensorMap map, map_lo;
-  if (encode(&map, type, 2, hi, gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-          CUDA_SUCCESS ||
-      encode(&map_lo, type, 2, lo, gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-          CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
+  const auto encode_map = [&](CUtensorMap* map, void* base) {
+    return encode(map, type, 2, base, gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  CUtensorMap map;
+  if (!encode_map(&map, hi)) return cudaErrorInvalidValue;
+  CUtensorMap map_lo = map;
+  if (split && !encode_map(&map_lo, lo)) return cudaErrorInvalidValue;
   // Kernel instances: fp32 tokens (8 epilogue warps), bf16 with 8, bf16 with
   // 16 (rows of at most kWideEpilogueMaxDim features).
   static std::atomic<uint64_t> attr_done[3] = {{0}, {0}, {0}};
