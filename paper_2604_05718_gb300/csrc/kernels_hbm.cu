@@ -311,19 +311,22 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
 // (C = 1, 2, 4 or 8, chosen by the launch) per image.  Every block takes a run
 // of consecutive rows, up to kScanElems per thread, and the blocks exchange
 // their counts through distributed shared memory, so that a run's IDs start
-// where the previous run's end.  The last image to finish turns the counts
-// into out_offsets.
+// where the previous run's end.  The pair average that follows turns the
+// counts into out_offsets.
 //
 // The kernel is bound by latency, not bytes: a row costs two dependent key
 // loads, and a block one barrier (two for a cluster).  One block per image,
 // 1024 rows at a time and three barriers a round, took 2.8 us for one image
 // of 1024 rows, 6.3 for 3136, 21.6 for 16384 and 7.6 for 24 images of up to
-// 4096; now 1.4, 2.7, 3.7 and 5.6.  64 images of 1024 rows take 3.6 us as
-// before: their last ticket and the offsets behind it.
+// 4096; now 1.4, 2.6, 3.7 and 3.2.  Offsets by the last image to finish (a
+// ticket, then the counts) took 1 to 2.3 us more of every batch: 64 images of
+// 1024 rows 3.7 us instead of 2.0.
 // ---------------------------------------------------------------------------
 constexpr int kScanThreads = 1024;
 constexpr int kScanElems = 4;
 constexpr int kScanMaxCluster = 8;
+// Images whose counts every block of the pair average adds up itself.
+constexpr int kStagedImages = 1024;
 
 __device__ __forceinline__ uint32_t scan_cluster_rank() {
   uint32_t r;
@@ -443,15 +446,11 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch,
     }
   }
   if (rank != 0) return;
-  if (batch == 1) {
-    if (threadIdx.x == 0) {
-      out_offsets[0] = 0;
-      out_offsets[1] = carry;
-    }
-    return;
-  }
+  if (threadIdx.x == 0) ws.count[b] = carry;
+  if (batch <= kStagedImages) return;
+  // More images than the pair average's blocks turn into offsets themselves:
+  // the last image to finish does it for all.
   if (threadIdx.x == 0) {
-    ws.count[b] = carry;
     // The ticket increment releases this image's count and, in the last
     // image's block, acquires all the others' (their increments came first).
     int prev;
@@ -461,8 +460,6 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch,
   __syncthreads();
   if (!is_last) return;
   // Counts -> out_offsets.  Their sum is at most the rows, which fit 32 bits.
-  // (One warp with four counts per lane, without barriers, was slower: this
-  // code runs once, so its length counts.)
   int acc = 0;
   for (int c0 = 0; c0 <= batch; c0 += kScanThreads) {
     const int idx = c0 + threadIdx.x;
@@ -478,35 +475,76 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch,
 // ---------------------------------------------------------------------------
 // Pair average + compaction (Eq. 2): one warp per output row.
 // ---------------------------------------------------------------------------
-template <int U>
+template <int U, bool ONE>
 __global__ void __launch_bounds__(kThreads) pair_average_kernel(const uint8_t* __restrict__ tokens,
                                                                 uint8_t* __restrict__ out,
                                                                 int batch, int64_t rows, int row_bytes,
-                                                                bool bf16, Workspace ws,
-                                                                const int64_t* __restrict__ out_offsets,
+                                                                bool bf16, Workspace ws, int64_t* out_offsets,
                                                                 bool spread) {
   MPM_TRACE_BEGIN(MPM_TRACE_PAIR_AVERAGE);
+  // First input and output row of every image.  Each block adds the counts up
+  // itself: one load and a scan, where searching finished offsets is a chain
+  // of dependent loads, which is what bounds few rows.
+  extern __shared__ int32_t offsets_s[];  // [2 batch + 1] when staged
+  __shared__ int32_t sh[32];
+  const bool staged = !ONE && batch <= kStagedImages;
+  int32_t* const out_s = offsets_s;             // [batch + 1]
+  int32_t* const in_s = offsets_s + batch + 1;  // [batch]
   wait_for_previous_grid();
   MPM_TRACE_WAITED();
+  int64_t total = 0;
+  int64_t lo = 1, hi = 0, in_base = 0;  // empty: the first row is always looked up
+  if (ONE) {
+    total = hi = ws.count[0];
+    lo = 0;
+    in_base = ws.soff[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      out_offsets[0] = 0;
+      out_offsets[1] = total;
+    }
+  } else if (staged) {
+    int acc = 0;
+    for (int base = 0; base < batch; base += kThreads) {
+      const int idx = base + static_cast<int>(threadIdx.x);
+      const int v = idx < batch ? ws.count[idx] : 0;
+      const int64_t in = idx < batch ? ws.soff[idx] : 0;
+      int sum;
+      const int incl = block_incl_sum<int>(v, sh, &sum);
+      if (idx < batch) {
+        in_s[idx] = static_cast<int32_t>(in);
+        out_s[idx] = acc + incl - v;
+      }
+      acc += sum;
+    }
+    if (threadIdx.x == 0) out_s[batch] = acc;
+    __syncthreads();
+    total = acc;
+    if (blockIdx.x == 0)
+      for (int idx = threadIdx.x; idx <= batch; idx += kThreads) out_offsets[idx] = out_s[idx];
+  } else {
+    total = clamp64(out_offsets[batch], 0, rows);
+  }
   const int lane = threadIdx.x & 31;
   const int64_t warp = warp_number(blockIdx.x, gridDim.x, spread);
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
   const int nvec = row_bytes >> 4;
-  int b = 0;
-  int64_t lo = 1, hi = 0, in_base = 0;  // empty: the first row is always looked up
-  int64_t total = INT64_MAX;  // known from the first look-up on
-  // A row's chain of dependent loads is what bounds few rows: the image
-  // search, its offsets, the pair, the tokens.  The total is loaded with the
-  // first image's offsets, not before them, and few rows spread over the SMs
-  // (1024 rows of 768 B: 3.6 -> 1.5 us).
   for (int64_t t = warp; t < total; t += nwarps) {
-    if (t >= hi || t < lo) {
-      b = find_image(out_offsets, batch, t);
-      lo = __ldg(out_offsets + b);
-      hi = __ldg(out_offsets + b + 1);
-      in_base = ws.soff[b];
-      total = clamp64(__ldg(out_offsets + batch), 0, rows);
-      if (t >= total) break;
+    if (!ONE && (t >= hi || t < lo)) {
+      if (staged) {
+        int b = 0, top = batch - 1;
+        while (b < top) {
+          const int mid = (b + top + 1) >> 1;
+          if (out_s[mid] <= t) b = mid; else top = mid - 1;
+        }
+        lo = out_s[b];
+        hi = out_s[b + 1];
+        in_base = in_s[b];
+      } else {
+        const int b = find_image(out_offsets, batch, t);
+        lo = out_offsets[b];
+        hi = out_offsets[b + 1];
+        in_base = ws.soff[b];
+      }
     }
     const int2 rep = ws.reps[in_base + (t - lo)];
     const bool pair = rep.y >= 0;
@@ -782,11 +820,21 @@ cudaError_t launch_mutual_compact(int batch, int64_t rows, int64_t chunk, const 
 
 cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch, int64_t rows,
                                 int dim, bool bf16, const Workspace& ws,
-                                const int64_t* out_offsets, int num_sms, cudaStream_t stream) {
+                                int64_t* out_offsets, int num_sms, cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
-  static const int per_sm = resident_per_sm(pair_average_kernel<4>, kThreads, 8);
+  // A single image needs no shared memory and no barriers (with them, one of
+  // 3136 rows took 1 us more a merge).
+  if (batch == 1) {
+    static const int per_sm = resident_per_sm(pair_average_kernel<4, true>, kThreads, 8);
+    const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm));
+    return launch_dependent(pair_average_kernel<4, true>, dim3(g.blocks), dim3(kThreads), 0, stream,
+                            static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch, rows,
+                            row_bytes, bf16, ws, out_offsets, g.spread);
+  }
+  static const int per_sm = resident_per_sm(pair_average_kernel<4, false>, kThreads, 8);
   const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm));
-  return launch_dependent(pair_average_kernel<4>, dim3(g.blocks), dim3(kThreads), 0, stream,
+  const size_t smem = batch <= kStagedImages ? (2 * static_cast<size_t>(batch) + 1) * sizeof(int32_t) : 0;
+  return launch_dependent(pair_average_kernel<4, false>, dim3(g.blocks), dim3(kThreads), smem, stream,
                           static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch, rows,
                           row_bytes, bf16, ws, out_offsets, g.spread);
 }

@@ -68,14 +68,15 @@ cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, in
                                  const Workspace& ws, int num_sms, cudaStream_t stream);
 AffinityTile pair_tile();
 
-// Mutual check, representative scan, per-image counts, output offsets.
+// Mutual check, representative scan, per-image counts (and, for very many
+// images, the output offsets).
 cudaError_t launch_mutual_compact(int batch, int64_t rows, int64_t chunk, const Workspace& ws, int32_t* out_map,
                                   int64_t* out_offsets, int num_sms, cudaStream_t stream);
 
-// Pair average + compaction into the packed output.
+// Output offsets, pair average + compaction into the packed output.
 cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch, int64_t rows,
                                 int dim, bool bf16, const Workspace& ws,
-                                const int64_t* out_offsets, int num_sms, cudaStream_t stream);
+                                int64_t* out_offsets, int num_sms, cudaStream_t stream);
 
 // Keys -> nearest neighbour index and cosine.
 cudaError_t launch_decode_nn(int batch, int64_t rows, const Workspace& ws, int32_t* out_nn,

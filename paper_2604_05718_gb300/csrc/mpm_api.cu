@@ -249,8 +249,8 @@ mpm_status merge_impl(const void* tokens, const int64_t* offsets, int32_t batch,
     e = mpm::launch_mutual_compact(batch, rows, chunk, ws, out_map, out_offsets, sms, s);
   }
   if (e != cudaSuccess || !mark(5) || !mark(6)) return MPM_ERR_CUDA;
-  if (rows > 0) {
-    const Range r("mpm.pair_average");
+  {
+    const Range r("mpm.pair_average");  // writes out_offsets too, so also without rows
     e = mpm::launch_pair_average(tokens, out_tokens, batch, rows, dim, bf16, ws, out_offsets, sms, s);
     if (e != cudaSuccess) return MPM_ERR_CUDA;
   }

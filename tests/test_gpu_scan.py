@@ -42,6 +42,8 @@ def mpm():
     ([32769 + 2048], 256),            # a second round with few rows
     ([12000] + [5] * 40, 512),        # one long image among short ones: rounds of one block
     ([3, 1, 2] * 400, 0),             # more images than a block has threads
+    ([2] * 1024, 0),                  # the pair average adds up to 1024 counts itself
+    ([2, 1, 0] * 341 + [3, 3], 0),    # 1025 images: the scan does
     ([2300] * 80, 256),               # too many images for two blocks each
     ([700], 1 << 40),                 # a chunk longer than any image
 ])
