@@ -44,6 +44,7 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 L2_FLUSH_BYTES = 256 << 20
 KERNELS_PER_MERGE = 4
+SMALL_MERGE_ROWS, SMALL_MERGE_IMAGES = 1024, 256
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "affinity_pair_traffic.txt")
 # The sources the affinity kernel is compiled from; the traffic record holds
 # a hash of their concatenation.
@@ -377,8 +378,9 @@ class Step:
                       if self.two else None)
 
     def launches(self) -> int:
-        """Kernels of the library launched by one step."""
-        return 2 * KERNELS_PER_MERGE + 1 if self.two else KERNELS_PER_MERGE + 1
+        """Kernels of the library launched by one step (a merge of few rows takes its last two steps in one)."""
+        per_merge = KERNELS_PER_MERGE - (self.batch.rows <= SMALL_MERGE_ROWS and self.batch.batch <= SMALL_MERGE_IMAGES)
+        return 2 * per_merge + 1 if self.two else per_merge + 1
 
     def run(self, ev: StepEvents, host_in=None, host_out=None, per_kernel=False):
         """One step; per_kernel adds CUDA events between the kernels (which

@@ -78,6 +78,12 @@ cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch,
                                 int dim, bool bf16, const Workspace& ws,
                                 int64_t* out_offsets, int num_sms, cudaStream_t stream);
 
+// The two steps above in one launch, for batches that merge_tail_fits allows.
+bool merge_tail_fits(int batch, int64_t rows);
+cudaError_t launch_merge_tail(const void* tokens, void* out_tokens, int batch, int64_t rows, int dim, bool bf16,
+                              int64_t chunk, const Workspace& ws, int32_t* out_map, int64_t* out_offsets, int num_sms,
+                              cudaStream_t stream);
+
 // Keys -> nearest neighbour index and cosine.
 cudaError_t launch_decode_nn(int batch, int64_t rows, const Workspace& ws, int32_t* out_nn,
                              float* out_score, int num_sms, cudaStream_t stream);

@@ -243,6 +243,13 @@ mpm_status merge_impl(const void* tokens, const int64_t* offsets, int32_t batch,
     e = launch_affinity(algo, tokens, batch, rows, dim, bf16, chunk, ws, sms, s);
     if (e != cudaSuccess) return MPM_ERR_CUDA;
   }
+  // Small batches take both remaining steps in one launch, unless the caller
+  // times them one by one.
+  if (stage_events == nullptr && mpm::merge_tail_fits(batch, rows)) {
+    const Range r("mpm.merge_tail");
+    return cuda_status(mpm::launch_merge_tail(tokens, out_tokens, batch, rows, dim, bf16, chunk, ws, out_map,
+                                              out_offsets, sms, s));
+  }
   if (!mark(3) || !mark(4)) return MPM_ERR_CUDA;
   {
     const Range r("mpm.mutual_scan");
