@@ -17,19 +17,6 @@ __device__ __forceinline__ int64_t clamp64(int64_t v, int64_t lo, int64_t hi) {
   return v < lo ? lo : (v > hi ? hi : v);
 }
 
-// Finds the image of row p, reusing the previous answer when p is still in
-// the same image (rows are visited in increasing order by each warp).
-struct ImageCursor {
-  int b = 0;
-  int64_t lo = 1, hi = 0;  // empty: forces the first search
-  __device__ __forceinline__ void locate(const int64_t* off, int batch, int64_t p) {
-    if (p >= lo && p < hi) return;
-    b = find_image(off, batch, p);
-    lo = __ldg(off + b);
-    hi = __ldg(off + b + 1);
-  }
-};
-
 // ---------------------------------------------------------------------------
 // Prep: status reset, offsets sanitisation + work plan (block 0), inverse
 // row norms and key reset (all other blocks).  Large batches are bound by
@@ -768,7 +755,40 @@ RowDiv row_div(int row_bytes) {
   return {nvec, nvec == 1 ? 0x80000000u : 0x80000000u / nvec + 1u};
 }
 
-template <int U, bool COMPOSE>
+// An array of offsets in global memory, or its copy in shared memory.
+template <bool STAGED>
+struct Offsets {
+  const int64_t* p;
+  __device__ __forceinline__ int64_t operator[](int k) const { return STAGED ? p[k] : __ldg(p + k); }
+};
+
+// Finds the image of row p, reusing the previous answer when p is still in
+// the same image (rows are visited in increasing order by each warp).
+template <bool STAGED>
+struct ImageCursor {
+  int b = 0;
+  int64_t lo = 1, hi = 0;  // empty: forces the first search
+  __device__ __forceinline__ void locate(const Offsets<STAGED>& off, int batch, int64_t p) {
+    if (p >= lo && p < hi) return;
+    int last = batch - 1;
+    b = 0;
+    while (b < last) {
+      const int mid = (b + last + 1) >> 1;
+      if (off[mid] <= p) b = mid; else last = mid - 1;
+    }
+    lo = off[b];
+    hi = off[b + 1];
+  }
+};
+
+// Images from which on every block copies their offsets to shared memory: a
+// search in global memory is a chain of dependent loads (64 images of 1024 x
+// 768 bf16: 22.9 instead of 21.6 us, 32 of 1024 x 384: 8.1 instead of 7.5),
+// but for a few images the copy and its barrier take longer (3 images: 1.7
+// against 2.0 us).  The upper bound keeps the copy within 6 KiB.
+constexpr int kStagedFrom = 9, kStagedTo = 256;
+
+template <int U, bool COMPOSE, bool STAGED>
 __global__ void __launch_bounds__(kThreads) gather_kernel(const uint8_t* __restrict__ merged,
                                                           const int64_t* __restrict__ moff,
                                                           int64_t merged_rows,
@@ -782,13 +802,26 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const uint8_t* __restr
   MPM_TRACE_BEGIN(MPM_TRACE_GATHER);
   wait_for_previous_grid();
   MPM_TRACE_WAITED();
+  Offsets<STAGED> grid_at{goff}, merged_at{moff}, mid_at{off1};
+  if constexpr (STAGED) {
+    extern __shared__ int64_t offs_s[];  // goff, moff and (COMPOSE) off1, [batch + 1] each
+    for (int k = threadIdx.x; k <= batch; k += kThreads) {
+      offs_s[k] = goff[k];
+      offs_s[batch + 1 + k] = moff[k];
+      if (COMPOSE) offs_s[2 * (batch + 1) + k] = off1[k];
+    }
+    __syncthreads();
+    grid_at.p = offs_s;
+    merged_at.p = offs_s + batch + 1;
+    mid_at.p = offs_s + 2 * (batch + 1);
+  }
   const int lane = threadIdx.x & 31;
   // Neighbouring runs go to neighbouring blocks, so that few rows still use
   // every SM.
   const int64_t warp = static_cast<int64_t>(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
-  const int64_t used = clamp64(goff[batch], 0, grid_rows);
-  ImageCursor cur;
+  const int64_t used = clamp64(grid_at[batch], 0, grid_rows);
+  ImageCursor<STAGED> cur;
   for (int64_t p0 = warp * per_warp; p0 < used; p0 += nwarps * per_warp) {
     // Lane l resolves grid row p0 + l.
     const int64_t p = p0 + lane;
@@ -796,12 +829,12 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const uint8_t* __restr
     int32_t src = -1;  // merged row to copy, -1 = none (zero row)
     if (lane < nrows) {
       int32_t m = map[p];
-      cur.locate(goff, batch, p);
-      const int64_t mlo = __ldg(moff + cur.b), mhi = __ldg(moff + cur.b + 1);
+      cur.locate(grid_at, batch, p);
+      const int64_t mlo = merged_at[cur.b], mhi = merged_at[cur.b + 1];
       bool ok = p >= cur.lo && p < cur.hi;
       if (COMPOSE) {
         // Stage-1 index of this grid row, then its stage-2 (merged) index.
-        const int64_t lo1 = __ldg(off1 + cur.b), hi1 = __ldg(off1 + cur.b + 1);
+        const int64_t lo1 = mid_at[cur.b], hi1 = mid_at[cur.b + 1];
         ok = ok && m >= 0 && m < hi1 - lo1 && lo1 >= 0 && lo1 + m < rows1;
         m = ok ? __ldg(map2 + lo1 + m) : -1;
       }
@@ -984,19 +1017,36 @@ cudaError_t launch_compose(const int32_t* map1, const int64_t* off0, int64_t row
                           map2, off1, rows1, batch, out, status);
 }
 
+namespace {
+// Gather, or composition and gather (map2 and off1 given).
+template <bool COMPOSE>
+cudaError_t launch_gather_kernel(const void* merged, const int64_t* moff, int64_t merged_rows, const int32_t* map,
+                                 const int64_t* goff, int64_t grid_rows, const int32_t* map2, const int64_t* off1,
+                                 int64_t rows1, int32_t* out_map, int batch, int dim, bool bf16, void* out,
+                                 int32_t* status, int num_sms, cudaStream_t stream) {
+  const int row_bytes = dim * (bf16 ? 2 : 4);
+  const auto launch = [&](auto kernel, int per_sm, size_t smem) {
+    const GatherShape g = gather_shape(grid_rows, grid_for(num_sms, per_sm));
+    return launch_dependent(kernel, dim3(g.grid), dim3(kThreads), smem, stream, static_cast<const uint8_t*>(merged),
+                            moff, merged_rows, map, goff, grid_rows, map2, off1, rows1, out_map, batch,
+                            row_div(row_bytes), g.per_warp, static_cast<uint8_t*>(out), status);
+  };
+  if (batch >= kStagedFrom && batch <= kStagedTo) {
+    static const int per_sm = resident_per_sm(gather_kernel<kGatherVecs, COMPOSE, true>, kThreads, 8);
+    return launch(gather_kernel<kGatherVecs, COMPOSE, true>, per_sm,
+                  (COMPOSE ? 3 : 2) * sizeof(int64_t) * (static_cast<size_t>(batch) + 1));
+  }
+  static const int per_sm = resident_per_sm(gather_kernel<kGatherVecs, COMPOSE, false>, kThreads, 8);
+  return launch(gather_kernel<kGatherVecs, COMPOSE, false>, per_sm, 0);
+}
+}  // namespace
+
 cudaError_t launch_gather(const void* merged, const int64_t* moff, int64_t merged_rows,
                           const int32_t* map, const int64_t* goff, int64_t grid_rows, int batch,
                           int dim, bool bf16, void* out, int32_t* status, int num_sms,
                           cudaStream_t stream) {
-  const int row_bytes = dim * (bf16 ? 2 : 4);
-  auto kernel = gather_kernel<kGatherVecs, false>;
-  static const int per_sm = resident_per_sm(kernel, kThreads, 8);
-  const GatherShape g = gather_shape(grid_rows, grid_for(num_sms, per_sm));
-  return launch_dependent(kernel, dim3(g.grid), dim3(kThreads), 0, stream, static_cast<const uint8_t*>(merged), moff,
-                          merged_rows, map, goff, grid_rows, static_cast<const int32_t*>(nullptr),
-                          static_cast<const int64_t*>(nullptr), static_cast<int64_t>(0),
-                          static_cast<int32_t*>(nullptr), batch, row_div(row_bytes), g.per_warp,
-                          static_cast<uint8_t*>(out), status);
+  return launch_gather_kernel<false>(merged, moff, merged_rows, map, goff, grid_rows, nullptr, nullptr, 0, nullptr,
+                                     batch, dim, bf16, out, status, num_sms, stream);
 }
 
 cudaError_t launch_compose_gather(const void* merged, const int64_t* moff, int64_t merged_rows,
@@ -1004,13 +1054,8 @@ cudaError_t launch_compose_gather(const void* merged, const int64_t* moff, int64
                                   const int32_t* map2, const int64_t* off1, int64_t rows1, int batch, int dim,
                                   bool bf16, void* out, int32_t* out_map, int32_t* status, int num_sms,
                                   cudaStream_t stream) {
-  const int row_bytes = dim * (bf16 ? 2 : 4);
-  auto kernel = gather_kernel<kGatherVecs, true>;
-  static const int per_sm = resident_per_sm(kernel, kThreads, 8);
-  const GatherShape g = gather_shape(rows0, grid_for(num_sms, per_sm));
-  return launch_dependent(kernel, dim3(g.grid), dim3(kThreads), 0, stream, static_cast<const uint8_t*>(merged), moff,
-                          merged_rows, map1, off0, rows0, map2, off1, rows1, out_map, batch, row_div(row_bytes),
-                          g.per_warp, static_cast<uint8_t*>(out), status);
+  return launch_gather_kernel<true>(merged, moff, merged_rows, map1, off0, rows0, map2, off1, rows1, out_map, batch,
+                                    dim, bf16, out, status, num_sms, stream);
 }
 
 }  // namespace mpm

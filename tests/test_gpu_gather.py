@@ -42,6 +42,10 @@ def offsets(counts):
     (torch.float32, 16384, [19]),                  # 4096, the longest row
     (torch.bfloat16, 64, [152 * 3 * 8 * 8 + 1]),   # about one round of runs
     (torch.bfloat16, 16, [40000, 39999]),          # several rounds
+    (torch.bfloat16, 40, [9, 0, 70, 1, 0, 0, 33, 2]),            # 8 images: offsets searched in place
+    (torch.float32, 40, [0, 9, 0, 70, 1, 0, 33, 2, 500]),        # 9: from shared memory
+    (torch.bfloat16, 8, [3] * 256),
+    (torch.bfloat16, 8, [3, 1, 0] * 85 + [4, 5]),                # 257: in place again
 ])
 def test_gather_equals_indexing(mpm, dtype, dim, counts):
     gen = torch.Generator(device=DEV).manual_seed(5)
