@@ -880,20 +880,6 @@ RowGrid row_grid(int64_t items, int wave) {
   return {blocks > 1 ? static_cast<int>(blocks) : 1, true};
 }
 
-// Blocks and rows per warp of the gather for `rows` grid rows: at most one
-// wave of blocks, and rows dealt evenly over its warps (at most kGatherRows a
-// warp and round).
-struct GatherShape {
-  int grid, per_warp;
-};
-GatherShape gather_shape(int64_t rows, int wave) {
-  const int64_t warps = static_cast<int64_t>(wave) * (kThreads / 32);
-  const int64_t rounds = (rows + kGatherRows * warps - 1) / (kGatherRows * warps);
-  const int64_t per_warp = (rows + warps * rounds - 1) / (warps * rounds);
-  const int64_t need = (rows + per_warp * (kThreads / 32) - 1) / (per_warp * (kThreads / 32));
-  return {static_cast<int>(need < wave ? need : wave), static_cast<int>(per_warp)};
-}
-
 }  // namespace
 
 #ifdef MPM_TRACE
@@ -1026,7 +1012,7 @@ cudaError_t launch_gather_kernel(const void* merged, const int64_t* moff, int64_
                                  int32_t* status, int num_sms, cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
   const auto launch = [&](auto kernel, int per_sm, size_t smem) {
-    const GatherShape g = gather_shape(grid_rows, grid_for(num_sms, per_sm));
+    const RunShape g = run_shape(grid_rows, grid_for(num_sms, per_sm), kThreads / 32, kGatherRows);
     return launch_dependent(kernel, dim3(g.grid), dim3(kThreads), smem, stream, static_cast<const uint8_t*>(merged),
                             moff, merged_rows, map, goff, grid_rows, map2, off1, rows1, out_map, batch,
                             row_div(row_bytes), g.per_warp, static_cast<uint8_t*>(out), status);
