@@ -135,7 +135,9 @@ MPM_API mpm_status mpm_merge(const void* tokens, const int64_t* offsets, int32_t
  * and stage_events[2k+1] just after it, for k = 0 row norms and work plan,
  * 1 affinity + arg max (Eq. 1, Algorithm 1 step 3), 2 mutual check and
  * left-to-right compaction scan (steps 4-6), 3 pair average (Eq. 2).
- * Otherwise identical to mpm_merge (which is this call with NULL).
+ * Otherwise identical to mpm_merge (which is this call with NULL; without
+ * events, steps 2 and 3 of a small batch share one launch, recorded as
+ * MPM_TRACE_MUTUAL in a traced library).
  */
 MPM_API mpm_status mpm_merge_timed(const void* tokens, const int64_t* offsets, int32_t batch,
                                    int64_t rows, int32_t dim, mpm_dtype dtype, void* out_tokens,

@@ -462,36 +462,9 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch,
 // ---------------------------------------------------------------------------
 // Pair average + compaction (Eq. 2): one warp per output row.
 // ---------------------------------------------------------------------------
-// Output row t: input row `first`, averaged with input row `second` if it is
-// a pair (otherwise second = first).  All loads of a pass are issued before
-// any store.
-template <int U>
-__device__ __forceinline__ void average_row(const uint8_t* __restrict__ tokens, uint8_t* __restrict__ out,
-                                            int64_t first, int64_t second, bool pair, int64_t t, int row_bytes,
-                                            bool bf16) {
-  const int lane = threadIdx.x & 31, nvec = row_bytes >> 4;
-  const uint4* a = reinterpret_cast<const uint4*>(tokens + first * row_bytes);
-  const uint4* p = reinterpret_cast<const uint4*>(tokens + second * row_bytes);
-  uint4* dst = reinterpret_cast<uint4*>(out + t * row_bytes);
-  for (int v0 = lane; v0 < nvec; v0 += 32 * U) {
-    uint4 va[U], vb[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int v = v0 + 32 * u;
-      if (v < nvec) {
-        va[u] = __ldcs(a + v);
-        if (pair) vb[u] = __ldcs(p + v);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int v = v0 + 32 * u;
-      if (v < nvec) dst[v] = pair ? avg16(va[u], vb[u], bf16) : va[u];
-    }
-  }
-}
-
-template <int U, bool ONE>
+// R consecutive output rows at a time, U vectors of each in flight per lane:
+// all loads of a pass are issued before any store.
+template <int U, int R, bool ONE>
 __global__ void __launch_bounds__(kThreads) pair_average_kernel(const uint8_t* __restrict__ tokens,
                                                                 uint8_t* __restrict__ out,
                                                                 int batch, int64_t rows, int row_bytes,
@@ -542,27 +515,58 @@ __global__ void __launch_bounds__(kThreads) pair_average_kernel(const uint8_t* _
   }
   const int64_t warp = warp_number(blockIdx.x, gridDim.x, spread);
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
-  for (int64_t t = warp; t < total; t += nwarps) {
-    if (!ONE && (t >= hi || t < lo)) {
-      if (staged) {
-        int b = 0, top = batch - 1;
-        while (b < top) {
-          const int mid = (b + top + 1) >> 1;
-          if (out_s[mid] <= t) b = mid; else top = mid - 1;
+  const int lane = threadIdx.x & 31, nvec = row_bytes >> 4;
+  for (int64_t t0 = warp * R; t0 < total; t0 += nwarps * R) {
+    const uint4* a[R];
+    const uint4* p[R];
+    bool pair[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int64_t t = t0 + r < total ? t0 + r : t0;
+      if (!ONE && (t >= hi || t < lo)) {
+        if (staged) {
+          int b = 0, top = batch - 1;
+          while (b < top) {
+            const int mid = (b + top + 1) >> 1;
+            if (out_s[mid] <= t) b = mid; else top = mid - 1;
+          }
+          lo = out_s[b];
+          hi = out_s[b + 1];
+          in_base = in_s[b];
+        } else {
+          const int b = find_image(out_offsets, batch, t);
+          lo = out_offsets[b];
+          hi = out_offsets[b + 1];
+          in_base = ws.soff[b];
         }
-        lo = out_s[b];
-        hi = out_s[b + 1];
-        in_base = in_s[b];
-      } else {
-        const int b = find_image(out_offsets, batch, t);
-        lo = out_offsets[b];
-        hi = out_offsets[b + 1];
-        in_base = ws.soff[b];
       }
+      const int2 rep = ws.reps[in_base + (t - lo)];
+      pair[r] = rep.y >= 0;
+      a[r] = reinterpret_cast<const uint4*>(tokens + (in_base + rep.x) * row_bytes);
+      p[r] = reinterpret_cast<const uint4*>(tokens + (in_base + (pair[r] ? rep.y : rep.x)) * row_bytes);
     }
-    const int2 rep = ws.reps[in_base + (t - lo)];
-    const bool pair = rep.y >= 0;
-    average_row<U>(tokens, out, in_base + rep.x, in_base + (pair ? rep.y : rep.x), pair, t, row_bytes, bf16);
+    uint4* dst = reinterpret_cast<uint4*>(out + t0 * row_bytes);
+    for (int v0 = lane; v0 < nvec; v0 += 32 * U) {
+      uint4 va[R][U], vb[R][U];
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int v = v0 + 32 * u;
+          if (v < nvec) {
+            va[r][u] = __ldcs(a[r] + v);
+            if (pair[r]) vb[r][u] = __ldcs(p[r] + v);
+          }
+        }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int v = v0 + 32 * u;
+          if (v < nvec && t0 + r < total)
+            dst[static_cast<int64_t>(r) * nvec + v] = pair[r] ? avg16(va[r][u], vb[r][u], bf16) : va[r][u];
+        }
+    }
   }
 }
 
@@ -578,6 +582,35 @@ __global__ void __launch_bounds__(kThreads) pair_average_kernel(const uint8_t* _
 constexpr int kTailElems = 4;
 constexpr int kTailRows = kTailElems * kThreads;
 constexpr int kTailImages = kThreads;
+
+// Output row t: input row `first`, averaged with input row `second` if it is
+// a pair (otherwise second = first).  All loads of a pass are issued before
+// any store.
+template <int U>
+__device__ __forceinline__ void average_row(const uint8_t* __restrict__ tokens, uint8_t* __restrict__ out,
+                                            int64_t first, int64_t second, bool pair, int64_t t, int row_bytes,
+                                            bool bf16) {
+  const int lane = threadIdx.x & 31, nvec = row_bytes >> 4;
+  const uint4* a = reinterpret_cast<const uint4*>(tokens + first * row_bytes);
+  const uint4* p = reinterpret_cast<const uint4*>(tokens + second * row_bytes);
+  uint4* dst = reinterpret_cast<uint4*>(out + t * row_bytes);
+  for (int v0 = lane; v0 < nvec; v0 += 32 * U) {
+    uint4 va[U], vb[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int v = v0 + 32 * u;
+      if (v < nvec) {
+        va[u] = __ldcs(a + v);
+        if (pair) vb[u] = __ldcs(p + v);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int v = v0 + 32 * u;
+      if (v < nvec) dst[v] = pair ? avg16(va[u], vb[u], bf16) : va[u];
+    }
+  }
+}
 
 __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __restrict__ tokens,
                                                               uint8_t* __restrict__ out, int batch, int rows,
@@ -962,18 +995,27 @@ cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch,
   // A single image needs no shared memory and no barriers (with them, one of
   // 3136 rows took 1 us more a merge).
   if (batch == 1) {
-    static const int per_sm = resident_per_sm(pair_average_kernel<4, true>, kThreads, 8);
+    static const int per_sm = resident_per_sm(pair_average_kernel<4, 1, true>, kThreads, 8);
     const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm));
-    return launch_dependent(pair_average_kernel<4, true>, dim3(g.blocks), dim3(kThreads), 0, stream,
+    return launch_dependent(pair_average_kernel<4, 1, true>, dim3(g.blocks), dim3(kThreads), 0, stream,
                             static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch, rows,
                             row_bytes, bf16, ws, out_offsets, g.spread);
   }
-  static const int per_sm = resident_per_sm(pair_average_kernel<4, false>, kThreads, 8);
-  const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm));
-  const size_t smem = batch <= kStagedImages ? (2 * static_cast<size_t>(batch) + 1) * sizeof(int32_t) : 0;
-  return launch_dependent(pair_average_kernel<4, false>, dim3(g.blocks), dim3(kThreads), smem, stream,
-                          static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch, rows,
-                          row_bytes, bf16, ws, out_offsets, g.spread);
+  const auto launch = [&](auto kernel, int per_sm, int warp_rows) {
+    const RowGrid g = row_grid((rows + warp_rows - 1) / warp_rows, grid_for(num_sms, per_sm));
+    const size_t smem = batch <= kStagedImages ? (2 * static_cast<size_t>(batch) + 1) * sizeof(int32_t) : 0;
+    return launch_dependent(kernel, dim3(g.blocks), dim3(kThreads), smem, stream, static_cast<const uint8_t*>(tokens),
+                            static_cast<uint8_t*>(out_tokens), batch, rows, row_bytes, bf16, ws, out_offsets,
+                            g.spread);
+  };
+  // Rows of at most 64 vectors go in pairs: one row of 768 B left more than
+  // half of the four load slots empty (32768 rows: 10.4 us, in pairs 8.3).
+  if (row_bytes <= 1024) {
+    static const int per_sm = resident_per_sm(pair_average_kernel<2, 2, false>, kThreads, 8);
+    return launch(pair_average_kernel<2, 2, false>, per_sm, 2);
+  }
+  static const int per_sm = resident_per_sm(pair_average_kernel<4, 1, false>, kThreads, 8);
+  return launch(pair_average_kernel<4, 1, false>, per_sm, 1);
 }
 
 bool merge_tail_fits(int batch, int64_t rows) { return rows > 0 && rows <= kTailRows && batch <= kTailImages; }

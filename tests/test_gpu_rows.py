@@ -45,6 +45,13 @@ def mpm():
     ("bf16", 16, [5] * 256, 0),
     ("bf16", 16, [4, 0, 3] * 90, 17),
     ("bf16", 64, [300] * 20, 9000),           # more than a wave of rows, a third of them used
+    # Capacity past 1024 rows: the pair average in its own launch, rows in pairs up to 1 KiB.
+    ("bf16", 8, [1], 1100),
+    ("bf16", 512, [64, 1], 1100),
+    ("bf16", 520, [101], 1000),
+    ("f32", 256, [33, 0, 2], 1200),
+    ("f32", 260, [34], 1200),
+    ("bf16", 1024, [31, 31], 1000),
 ])
 def test_merge_row_classes(mpm, dtype, dim, counts, spare):
     batch = make_custom(counts, dim, dtype, seed=91 + dim)
