@@ -1008,11 +1008,22 @@ cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch,
                             static_cast<uint8_t*>(out_tokens), batch, rows, row_bytes, bf16, ws, out_offsets,
                             g.spread);
   };
-  // Rows of at most 64 vectors go in pairs: one row of 768 B left more than
-  // half of the four load slots empty (32768 rows: 10.4 us, in pairs 8.3).
+  // Rows and vectors per warp and round by the row's length, so that few load
+  // slots are empty (1 x 4 for every length: 32768 rows of 768 B 10.4 us, by
+  // twos 8.3; passes of two merges of 256 x 512 rows of 256 B 140.5 us with 2 x
+  // 2, 128.6 with 4 x 1, of 64 x 1024 rows of 1.5 KiB 197.6 with 1 x 4, 196.4
+  // with 2 x 3; 2 x 4 for 2 KiB was slower, 196.1 instead of 192.2).
+  if (row_bytes <= 512) {
+    static const int per_sm = resident_per_sm(pair_average_kernel<1, 4, false>, kThreads, 8);
+    return launch(pair_average_kernel<1, 4, false>, per_sm, 4);
+  }
   if (row_bytes <= 1024) {
     static const int per_sm = resident_per_sm(pair_average_kernel<2, 2, false>, kThreads, 8);
     return launch(pair_average_kernel<2, 2, false>, per_sm, 2);
+  }
+  if (row_bytes <= 1536) {
+    static const int per_sm = resident_per_sm(pair_average_kernel<3, 2, false>, kThreads, 8);
+    return launch(pair_average_kernel<3, 2, false>, per_sm, 2);
   }
   static const int per_sm = resident_per_sm(pair_average_kernel<4, 1, false>, kThreads, 8);
   return launch(pair_average_kernel<4, 1, false>, per_sm, 1);

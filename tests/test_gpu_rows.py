@@ -45,9 +45,14 @@ def mpm():
     ("bf16", 16, [5] * 256, 0),
     ("bf16", 16, [4, 0, 3] * 90, 17),
     ("bf16", 64, [300] * 20, 9000),           # more than a wave of rows, a third of them used
-    # Capacity past 1024 rows: the pair average in its own launch, rows in pairs up to 1 KiB.
+    # Capacity past 1024 rows: the pair average in its own launch, 4, 2 or 1 rows at a time.
     ("bf16", 8, [1], 1100),
+    ("bf16", 256, [66, 1], 1100),
+    ("bf16", 264, [35, 0, 1], 1100),
     ("bf16", 512, [64, 1], 1100),
+    ("bf16", 768, [45], 1100),
+    ("bf16", 776, [45], 1100),
+    ("f32", 64, [700, 333, 2, 1], 40),
     ("bf16", 520, [101], 1000),
     ("f32", 256, [33, 0, 2], 1200),
     ("f32", 260, [34], 1200),
