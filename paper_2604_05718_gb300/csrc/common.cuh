@@ -53,23 +53,6 @@ inline int resident_per_sm(void (*kernel)(Params...), int threads, int cap) {
 }
 
 // ---------------------------------------------------------------------------
-// Row copies (gather, pad, unpad): a warp takes a run of consecutive rows and
-// copies them as one sequence of 16-byte vectors.
-// ---------------------------------------------------------------------------
-// Blocks and rows per warp for `rows` rows: at most `wave` blocks, and rows
-// dealt evenly over their warps (at most `most` of up to 32 a warp and round).
-struct RunShape {
-  int grid, per_warp;
-};
-inline RunShape run_shape(int64_t rows, int wave, int block_warps, int most) {
-  const int64_t warps = static_cast<int64_t>(wave) * block_warps;
-  const int64_t rounds = (rows + most * warps - 1) / (most * warps);
-  const int64_t per_warp = (rows + warps * rounds - 1) / (warps * rounds);
-  const int64_t need = (rows + per_warp * block_warps - 1) / (per_warp * block_warps);
-  return {static_cast<int>(need < wave ? need : wave), static_cast<int>(per_warp)};
-}
-
-// ---------------------------------------------------------------------------
 // Device timeline (libmpm_trace.so only; see mpm_trace_read in mpm.h).  Each
 // translation unit with traced kernels keeps its own table, which
 // trace_copy_<unit> reads or resets from the host.

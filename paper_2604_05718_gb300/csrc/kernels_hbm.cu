@@ -913,6 +913,19 @@ RowGrid row_grid(int64_t items, int wave) {
   return {blocks > 1 ? static_cast<int>(blocks) : 1, true};
 }
 
+// Blocks and rows per warp for `rows` rows: at most `wave` blocks, and rows
+// dealt evenly over their warps (at most `most` of up to 32 a warp and round).
+struct RunShape {
+  int grid, per_warp;
+};
+RunShape run_shape(int64_t rows, int wave, int block_warps, int most) {
+  const int64_t warps = static_cast<int64_t>(wave) * block_warps;
+  const int64_t rounds = (rows + most * warps - 1) / (most * warps);
+  const int64_t per_warp = (rows + warps * rounds - 1) / (warps * rounds);
+  const int64_t need = (rows + per_warp * block_warps - 1) / (per_warp * block_warps);
+  return {static_cast<int>(need < wave ? need : wave), static_cast<int>(per_warp)};
+}
+
 }  // namespace
 
 #ifdef MPM_TRACE
