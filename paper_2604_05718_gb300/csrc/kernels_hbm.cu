@@ -205,10 +205,11 @@ __device__ __noinline__ RowScale odd_row_scale(const uint4* src, int nvec, float
   if (!__all_sync(0xFFFFFFFFu, finite))
     return {__int_as_float(0x7fc00000), 1.0f, 1.0f / fmaxf(sqrtf(sumsq), 1e-12f)};
   if (top == 0.f) return {1.0f, 1.0f, 1.0f / 1e-12f};
-  // Largest element to [2^7, 2^8): the norm of at most 2^14 elements stays
-  // below 2^15, and its square within fp32's range.
+  // Largest element to [2^7, 2^8) for the sum of squares: the norm of at most
+  // 2^14 elements stays below 2^15, and its square within fp32's range.
   const int e = 7 - ilogbf(top);
-  const float s1 = scalbnf(1.0f, e / 2), s2 = scalbnf(1.0f, e - e / 2);
+  const float s1 = scalbnf(1.0f, e / 2);
+  float s2 = scalbnf(1.0f, e - e / 2);
   float s = 0.f;
   for (int v = lane; v < nvec; v += 32) {
     const uint4 q = __ldg(src + v);
@@ -221,7 +222,13 @@ __device__ __noinline__ RowScale odd_row_scale(const uint4* src, int nvec, float
   }
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
-  return {s1, s2, 1.0f / fmaxf(sqrtf(s), 1e-12f * s1 * s2)};
+  // Then the norm to [2^14, 2^15), like every other row's, so that small
+  // elements keep as many bits.
+  const float norm = sqrtf(s);
+  const int up = 14 - ilogbf(norm);
+  const float inv = 1.0f / fmaxf(norm, 1e-12f * s1 * s2);
+  s2 = scalbnf(s2, up);
+  return {s1, s2, scalbnf(inv, -up)};
 }
 
 __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __restrict__ tokens,

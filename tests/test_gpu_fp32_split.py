@@ -69,6 +69,23 @@ def test_rows_of_any_magnitude(mpm):
     check(mpm, x.astype(np.float32))
 
 
+@pytest.mark.parametrize("scale", [1.0, 1e25, 1e-18])
+def test_small_features_of_rows_of_any_magnitude(mpm, scale):
+    """Rows with a feature of their own 2^18 times the others: their cosines come from the small
+    features alone.  The bound is relative: the split adds at most 2^-39 of a row's norm to each
+    feature's error, 2^-21 of a small one."""
+    rng = np.random.default_rng(7)
+    x = np.abs(rng.standard_normal((128, 96))) + 0.5
+    x[:, :4] = 0.0
+    for r in range(4):
+        x[r, r] = 2.0 ** 18
+    x = (x * scale).astype(np.float32)
+    xd = torch.from_numpy(x).to(DEV)
+    nn, score = (t.cpu().numpy()[:4] for t in mpm.nearest_neighbors(xd, torch.tensor([0, 128], device=DEV)))
+    s = oracle.cosine_affinity(x.astype(np.float64))[:4]
+    np.testing.assert_allclose(score, s[np.arange(4), nn], rtol=bound(96) + 2.0 ** -21, atol=0)
+
+
 def test_tiny_zero_and_non_finite_rows(mpm):
     """Rows below the norm's floor and zero rows score 0; a row with an infinity or NaN is nobody's neighbour."""
     rng = np.random.default_rng(4)
