@@ -5,6 +5,8 @@
 // warp per row; grids are sized from the SM count and loop over rows.
 #include <math.h>
 
+#include <type_traits>
+
 #include "mpm.h"
 #include "common.cuh"
 
@@ -231,6 +233,15 @@ __device__ __noinline__ RowScale odd_row_scale(const uint4* src, int nvec, float
   return {s1, s2, scalbnf(inv, -up)};
 }
 
+// Scale of a row from its sum of squares `sumsq` (the same in every lane).
+__device__ __forceinline__ RowScale row_scale(const uint4* src, int nvec, float sumsq) {
+  if (!(sumsq >= 0x1p-100f && sumsq <= 0x1p100f)) return odd_row_scale(src, nvec, sumsq);
+  const float norm = sqrtf(sumsq);
+  const int e = 14 - (static_cast<int>(__float_as_uint(norm) >> 23) - 127);
+  return {__uint_as_float(static_cast<uint32_t>(127 + e) << 23), 1.0f,
+          1.0f / fmaxf(norm, 1e-12f) * __uint_as_float(static_cast<uint32_t>(127 - e) << 23)};
+}
+
 __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __restrict__ tokens,
                                                               const int64_t* __restrict__ offsets, int batch,
                                                               int64_t rows, int dim, AffinityTile tile,
@@ -265,16 +276,7 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
     for (int v = lane + 32 * kSplitVecs; v < nvec; v += 32) s += sumsq16(__ldg(src + v), false);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
-    RowScale sc;
-    if (s >= 0x1p-100f && s <= 0x1p100f) {
-      const float norm = sqrtf(s);
-      const int e = 14 - (static_cast<int>(__float_as_uint(norm) >> 23) - 127);
-      sc.s1 = __uint_as_float(static_cast<uint32_t>(127 + e) << 23);
-      sc.s2 = 1.0f;
-      sc.inv = 1.0f / fmaxf(norm, 1e-12f) * __uint_as_float(static_cast<uint32_t>(127 - e) << 23);
-    } else {
-      sc = odd_row_scale(src, nvec, s);
-    }
+    const RowScale sc = row_scale(src, nvec, s);
     uint2* hi = reinterpret_cast<uint2*>(ws.split_hi) + r * stride;
     uint2* lo = reinterpret_cast<uint2*>(ws.split_lo) + r * stride;
 #pragma unroll
@@ -298,6 +300,96 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
       ws.keys[r] = 0ull;
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// fp32 rows that the fp16 parts cannot decide.  An element's parts are off by
+// at most 2^-39 of its row's norm (above), so a cosine by at most about 2^-38
+// sqrt(D).  That is no more than fp32's own rounding as long as the cosine is
+// above 2^-15 sqrt(D) in size.  A row whose best cosine is smaller (rows with
+// a huge feature of their own: its other features decide, and may have lost
+// bits or vanished) has its neighbour found again by fp32 products of its
+// run's tokens.  The kernels that read the keys of an fp32 call do that
+// first.  Ordinary tokens never come here: the best of 1000 random cosines is
+// about 3 / sqrt(D).  The check costs 0.2 us in the one-launch tail (one image
+// of 1024 x 192: 12.8 -> 13.0) and 0.2 to 1.1 in the scan (64 x 1024 x 192:
+// 80.5 -> 81.3; 256 x 256 x 32: 45.0 -> 46.1).  A kernel of its own before the
+// scan cost 1.6 to 2.4.
+// ---------------------------------------------------------------------------
+// Is the row's best cosine too small to trust?  Zero rows (all their cosines
+// are exactly 0) have the largest inverse norm, 1e12; every other row's, scaled,
+// is at most 2^-7 or so.
+// `limit` is 2^-15 sqrt(D).
+__device__ __forceinline__ bool undecided(unsigned long long key, float inv_norm, float limit) {
+  return (key != 0ull) & (inv_norm < 1e11f) & (fabsf(key_score(key) * inv_norm) < limit);
+}
+float decide_limit(int dim) { return 0x1p-15f * sqrtf(static_cast<float>(dim)); }
+
+// The best neighbour's packed key of row `row`, whose image starts at `base`,
+// among the n rows from base + first on.  Scores as the affinity kernel's:
+// products of the scaled rows times the neighbour's scaled inverse norm; ties
+// to the lowest index, NaN never wins.  Scores are compared 2^96 times as
+// large (at most 2^126), so that products of two rows' smallest features do
+// not vanish.  By a whole warp.
+__device__ __noinline__ unsigned long long exact_key(const float* tokens, int dim, int64_t base, int first, int n,
+                                                     int64_t row) {
+  const int lane = threadIdx.x & 31, nvec = dim >> 2;
+  const auto sum = [](float s) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+    return s;
+  };
+  const auto scale_of = [&](const uint4* x) {
+    float s = 0.f;
+#pragma unroll 1
+    for (int v = lane; v < nvec; v += 32) s += sumsq16(__ldg(x + v), false);
+    return row_scale(x, nvec, sum(s));
+  };
+  const uint4* const rows = reinterpret_cast<const uint4*>(tokens);
+  const uint4* const x = rows + row * nvec;
+  const RowScale a = scale_of(x);
+  float best = -INFINITY;
+  int at = -1;
+  for (int j = first; j < first + n; ++j) {
+    if (base + j == row) continue;
+    const uint4* const y = rows + (base + j) * nvec;
+    const RowScale b = scale_of(y);
+    float dot = 0.f;
+#pragma unroll 1
+    for (int v = lane; v < nvec; v += 32) {
+      const uint4 p = __ldg(x + v), q = __ldg(y + v);
+      const float* f = reinterpret_cast<const float*>(&p);
+      const float* g = reinterpret_cast<const float*>(&q);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        dot = fmaf(f[k] * a.s1 * a.s2 * 0x1p48f, g[k] * b.s1 * b.s2 * 0x1p48f, dot);
+    }
+    const float score = sum(dot) * b.inv;
+    if (score > best) {
+      best = score;
+      at = j;
+    }
+  }
+  return at < 0 ? 0ull : make_key(best * 0x1p-96f, at);
+}
+
+// `key`, or the row's key found again where `redo` is set.  Called by whole
+// warps, with the packed row of each lane.
+__device__ __noinline__ unsigned long long decide(bool redo, unsigned long long key, int64_t row, const float* tokens,
+                                                  int dim, int batch, int chunk, const int64_t* soff) {
+  const int lane = threadIdx.x & 31;
+  for (uint32_t left = __ballot_sync(0xFFFFFFFFu, redo); left != 0u; left &= left - 1u) {
+    const int src = __ffs(static_cast<int>(left)) - 1;
+    const int64_t r = __shfl_sync(0xFFFFFFFFu, row, src);
+    const int b = find_image(soff, batch, r);
+    const int64_t base = soff[b];
+    const int n = static_cast<int>(soff[b + 1] - base), local = static_cast<int>(r - base);
+    const int first = chunk > 0 ? (local / chunk) * chunk : 0;
+    const int len = chunk > 0 && n - first > chunk ? chunk : n - first;
+    const unsigned long long k = exact_key(tokens, dim, base, first, len, r);
+    if (lane == src) key = k;
+  }
+  return key;
 }
 
 // ---------------------------------------------------------------------------
@@ -346,8 +438,11 @@ __device__ __forceinline__ void store_to_rank(int32_t* p, uint32_t rank, int32_t
   asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
 }
 
-template <int ELEMS, bool CLUSTER>
-__global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch, int chunk, Workspace ws,
+// SPLIT: fp32 tokens, whose keys (a row's and its neighbour's) decide() checks
+// first.
+template <int ELEMS, bool CLUSTER, bool SPLIT>
+__global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(const float* __restrict__ tokens, int batch,
+                                                                      int dim, int chunk, float limit, Workspace ws,
                                                                       int32_t* __restrict__ out_map,
                                                                       int64_t* __restrict__ out_offsets) {
   MPM_TRACE_BEGIN(MPM_TRACE_MUTUAL);
@@ -378,12 +473,18 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch,
 #pragma unroll
     for (int e = 0; e < ELEMS; ++e) {
       const int64_t i = first + e * kScanThreads;
-      j[e] = (e < elems && i < n) ? key_index(ws.keys[base + i]) : -1;
+      const bool live = e < elems && i < n;
+      unsigned long long key = live ? ws.keys[base + i] : 0ull;
+      if constexpr (SPLIT) {
+        const float inv = live ? ws.inv_norm[base + i] : 0.f;
+        const bool redo = undecided(key, inv, limit);
+        if (__any_sync(0xFFFFFFFFu, redo)) key = decide(redo, key, base + i, tokens, dim, batch, chunk, ws.soff);
+      }
+      j[e] = key_index(key);
     }
 #pragma unroll
     for (int e = 0; e < ELEMS; ++e) {
       const int i = static_cast<int>(first + e * kScanThreads);  // used only where the row exists
-      bool rep = false;
       if (e < elems && first + e * kScanThreads < n) {
         // b(i) lies in i's chunk (the whole image without chunking), and only a
         // token alone in its chunk has none.
@@ -394,10 +495,18 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(int batch,
           report(ws.status, MPM_ERR_DEVICE_CHECK, static_cast<int32_t>(base + i));
           j[e] = -1;
         }
-        // (i, j) is a pair of P when b(j) = i as well (Section 3.2).
-        if (j[e] >= 0 && key_index(ws.keys[base + j[e]]) != i) j[e] = -1;
-        rep = j[e] < 0 || i < j[e];
       }
+      // (i, j) is a pair of P when b(j) = i as well (Section 3.2).
+      if constexpr (SPLIT) {
+        unsigned long long key = j[e] >= 0 ? ws.keys[base + j[e]] : 0ull;
+        const float inv = j[e] >= 0 ? ws.inv_norm[base + j[e]] : 0.f;
+        const bool redo = undecided(key, inv, limit);
+        if (__any_sync(0xFFFFFFFFu, redo)) key = decide(redo, key, base + j[e], tokens, dim, batch, chunk, ws.soff);
+        if (key_index(key) != i) j[e] = -1;
+      } else {
+        if (j[e] >= 0 && key_index(ws.keys[base + j[e]]) != i) j[e] = -1;
+      }
+      const bool rep = e < elems && first + e * kScanThreads < n && (j[e] < 0 || i < j[e]);
       reps[e] = __ballot_sync(0xFFFFFFFFu, rep);
       if (lane == 0) warp_count[buf][e][warp] = __popc(reps[e]);
     }
@@ -619,10 +728,12 @@ __device__ __forceinline__ void average_row(const uint8_t* __restrict__ tokens, 
   }
 }
 
+// SPLIT: fp32 tokens, whose keys decide() checks first.
+template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __restrict__ tokens,
                                                               uint8_t* __restrict__ out, int batch, int rows,
-                                                              int chunk, int row_bytes, bool bf16, Workspace ws,
-                                                              int32_t* __restrict__ out_map,
+                                                              int chunk, int row_bytes, bool bf16, float limit,
+                                                              Workspace ws, int32_t* __restrict__ out_map,
                                                               int64_t* __restrict__ out_offsets) {
   __shared__ int32_t first_s[kTailImages + 1];   // first input row of every image
   __shared__ int32_t start_s[kTailImages + 1];   // first output row of every image
@@ -635,14 +746,37 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
   MPM_TRACE_WAITED();
   const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
   int j[kTailElems], image[kTailElems];
+  [[maybe_unused]] bool redo = false;
+  {
+    unsigned long long key[kTailElems];
+    [[maybe_unused]] float inv[kTailElems];
 #pragma unroll
-  for (int e = 0; e < kTailElems; ++e) {
-    const int i = e * kThreads + tid;
-    j[e] = i < rows ? key_index(ws.keys[i]) : -1;
+    for (int e = 0; e < kTailElems; ++e) {
+      const int i = e * kThreads + tid;
+      key[e] = i < rows ? ws.keys[i] : 0ull;
+      if (SPLIT) inv[e] = i < rows ? ws.inv_norm[i] : 0.f;
+    }
+#pragma unroll
+    for (int e = 0; e < kTailElems; ++e) {
+      j[e] = key_index(key[e]);
+      if (SPLIT) redo |= undecided(key[e], inv[e], limit);
+    }
   }
   for (int idx = tid; idx <= batch; idx += kThreads) first_s[idx] = static_cast<int32_t>(ws.soff[idx]);
   __syncthreads();
   const int lead = first_s[0], used = first_s[batch];  // rows before the first image belong to none
+  if (SPLIT && __any_sync(0xFFFFFFFFu, redo)) {
+    // Rare: every block finds these rows' neighbours again for itself.
+    for (int e = 0; e < kTailElems; ++e) {
+      const int i = e * kThreads + tid;
+      const bool live = i >= lead && i < used;
+      const unsigned long long key = live ? ws.keys[i] : 0ull;
+      const int again = key_index(decide(live && undecided(key, ws.inv_norm[i], limit), key, i,
+                                         reinterpret_cast<const float*>(tokens), row_bytes >> 2, batch, chunk, ws.soff));
+#pragma unroll
+      for (int k = 0; k < kTailElems; ++k) j[k] = k == e && live ? again : j[k];
+    }
+  }
 #pragma unroll
   for (int e = 0; e < kTailElems; ++e) {
     const int i = e * kThreads + tid;
@@ -719,15 +853,24 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
 // ---------------------------------------------------------------------------
 // Keys -> nearest neighbour and cosine (test / diagnostics hook).
 // ---------------------------------------------------------------------------
-__global__ void decode_nn_kernel(int batch, int64_t rows, Workspace ws, int32_t* __restrict__ nn,
-                                 float* __restrict__ score) {
+template <bool SPLIT>
+__global__ void __launch_bounds__(kThreads, 4) decode_nn_kernel(const float* __restrict__ tokens, int batch, int dim,
+                                                                int chunk, float limit, Workspace ws,
+                                                                int32_t* __restrict__ nn, float* __restrict__ score) {
   wait_for_previous_grid();
   const int64_t used = ws.soff[batch];
-  for (int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < used;
-       g += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const unsigned long long k = ws.keys[g];
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t w0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + (threadIdx.x & ~31u); w0 < used; w0 += stride) {
+    const int64_t g = w0 + (threadIdx.x & 31);
+    unsigned long long k = g < used ? ws.keys[g] : 0ull;
+    const float inv = g < used ? ws.inv_norm[g] : 0.f;
+    if (SPLIT) {
+      const bool redo = undecided(k, inv, limit);
+      if (__any_sync(0xFFFFFFFFu, redo)) k = decide(redo, k, g, tokens, dim, batch, chunk, ws.soff);
+    }
+    if (g >= used) continue;
     nn[g] = key_index(k);
-    if (score != nullptr) score[g] = k == 0ull ? -INFINITY : key_score(k) * ws.inv_norm[g];
+    if (score != nullptr) score[g] = k == 0ull ? -INFINITY : key_score(k) * inv;
   }
 }
 
@@ -975,8 +1118,9 @@ cudaError_t launch_prep(const void* tokens, const int64_t* offsets, int batch, i
   return launch(prep_kernel<2, 4>, per_sm, 2);
 }
 
-cudaError_t launch_mutual_compact(int batch, int64_t rows, int64_t chunk, const Workspace& ws, int32_t* out_map,
-                                  int64_t* out_offsets, int num_sms, cudaStream_t stream) {
+cudaError_t launch_mutual_compact(const void* tokens, int batch, int64_t rows, int dim, int64_t chunk,
+                                  const Workspace& ws, int32_t* out_map, int64_t* out_offsets, int num_sms,
+                                  cudaStream_t stream) {
   // One block per 1024 rows of the mean image (the images' own lengths are on
   // the device), as long as all blocks run at once, two on an SM; longer
   // images take more rows per thread.
@@ -1003,9 +1147,14 @@ cudaError_t launch_mutual_compact(int batch, int64_t rows, int64_t chunk, const 
   // Four rows per thread, and the cluster's barriers, only where the mean
   // image needs them: they take 1 us more on images of 1024 rows.
   const bool more = static_cast<int64_t>(blocks) * kScanThreads < mean;
-  auto kernel = blocks > 1 ? (more ? mutual_compact_kernel<kScanElems, true> : mutual_compact_kernel<1, true>)
-                           : (more ? mutual_compact_kernel<kScanElems, false> : mutual_compact_kernel<1, false>);
-  return cudaLaunchKernelEx(&cfg, kernel, batch, chunk32, ws, out_map, out_offsets);
+  const auto pick = [&](auto split) {
+    constexpr bool S = decltype(split)::value;
+    return blocks > 1 ? (more ? mutual_compact_kernel<kScanElems, true, S> : mutual_compact_kernel<1, true, S>)
+                      : (more ? mutual_compact_kernel<kScanElems, false, S> : mutual_compact_kernel<1, false, S>);
+  };
+  const auto kernel = ws.split_hi != nullptr ? pick(std::true_type{}) : pick(std::false_type{});
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<const float*>(tokens), batch, dim, chunk32, decide_limit(dim), ws,
+                            out_map, out_offsets);
 }
 
 cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch, int64_t rows,
@@ -1054,19 +1203,28 @@ bool merge_tail_fits(int batch, int64_t rows) { return rows > 0 && rows <= kTail
 cudaError_t launch_merge_tail(const void* tokens, void* out_tokens, int batch, int64_t rows, int dim, bool bf16,
                               int64_t chunk, const Workspace& ws, int32_t* out_map, int64_t* out_offsets, int num_sms,
                               cudaStream_t stream) {
-  static const int per_sm = resident_per_sm(merge_tail_kernel, kThreads, 8);
-  const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm));
-  return launch_dependent(merge_tail_kernel, dim3(g.blocks), dim3(kThreads), 0, stream,
-                          static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch,
-                          static_cast<int>(rows), chunk < rows ? static_cast<int>(chunk) : 0,
-                          dim * (bf16 ? 2 : 4), bf16, ws, out_map, out_offsets);
+  const auto launch = [&](auto kernel, int per_sm) {
+    return launch_dependent(kernel, dim3(row_grid(rows, grid_for(num_sms, per_sm)).blocks), dim3(kThreads), 0, stream,
+                            static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch,
+                            static_cast<int>(rows), chunk < rows ? static_cast<int>(chunk) : 0,
+                            dim * (bf16 ? 2 : 4), bf16, decide_limit(dim), ws, out_map, out_offsets);
+  };
+  if (ws.split_hi != nullptr) {
+    static const int per_sm = resident_per_sm(merge_tail_kernel<true>, kThreads, 8);
+    return launch(merge_tail_kernel<true>, per_sm);
+  }
+  static const int per_sm = resident_per_sm(merge_tail_kernel<false>, kThreads, 8);
+  return launch(merge_tail_kernel<false>, per_sm);
 }
 
-cudaError_t launch_decode_nn(int batch, int64_t rows, const Workspace& ws, int32_t* out_nn,
-                             float* out_score, int num_sms, cudaStream_t stream) {
-  (void)rows;
-  return launch_dependent(decode_nn_kernel, dim3(grid_for(num_sms, 4)), dim3(kThreads), 0, stream, batch, rows, ws,
-                          out_nn, out_score);
+cudaError_t launch_decode_nn(const void* tokens, int batch, int64_t rows, int dim, int64_t chunk, const Workspace& ws,
+                             int32_t* out_nn, float* out_score, int num_sms, cudaStream_t stream) {
+  const auto launch = [&](auto kernel) {
+    return launch_dependent(kernel, dim3(grid_for(num_sms, 4)), dim3(kThreads), 0, stream,
+                            static_cast<const float*>(tokens), batch, dim,
+                            chunk < rows ? static_cast<int>(chunk) : 0, decide_limit(dim), ws, out_nn, out_score);
+  };
+  return ws.split_hi != nullptr ? launch(decode_nn_kernel<true>) : launch(decode_nn_kernel<false>);
 }
 
 cudaError_t launch_compose(const int32_t* map1, const int64_t* off0, int64_t rows0,

@@ -70,8 +70,9 @@ AffinityTile pair_tile();
 
 // Mutual check, representative scan, per-image counts (and, for very many
 // images, the output offsets).
-cudaError_t launch_mutual_compact(int batch, int64_t rows, int64_t chunk, const Workspace& ws, int32_t* out_map,
-                                  int64_t* out_offsets, int num_sms, cudaStream_t stream);
+cudaError_t launch_mutual_compact(const void* tokens, int batch, int64_t rows, int dim, int64_t chunk,
+                                  const Workspace& ws, int32_t* out_map, int64_t* out_offsets, int num_sms,
+                                  cudaStream_t stream);
 
 // Output offsets, pair average + compaction into the packed output.
 cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch, int64_t rows,
@@ -85,8 +86,8 @@ cudaError_t launch_merge_tail(const void* tokens, void* out_tokens, int batch, i
                               cudaStream_t stream);
 
 // Keys -> nearest neighbour index and cosine.
-cudaError_t launch_decode_nn(int batch, int64_t rows, const Workspace& ws, int32_t* out_nn,
-                             float* out_score, int num_sms, cudaStream_t stream);
+cudaError_t launch_decode_nn(const void* tokens, int batch, int64_t rows, int dim, int64_t chunk, const Workspace& ws,
+                             int32_t* out_nn, float* out_score, int num_sms, cudaStream_t stream);
 
 cudaError_t launch_compose(const int32_t* map1, const int64_t* off0, int64_t rows0,
                            const int32_t* map2, const int64_t* off1, int64_t rows1, int batch,

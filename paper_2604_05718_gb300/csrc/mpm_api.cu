@@ -170,7 +170,6 @@ mpm_status run_affinity(const void* tokens, const int64_t* offsets, int32_t batc
                         mpm_dtype dtype, mpm_nn_algo algo, int64_t chunk, const Workspace& ws_all,
                         cudaStream_t stream) {
   const bool bf16 = dtype == MPM_BF16;
-  if (algo == MPM_NN_AUTO) algo = default_algo(dtype);
   const bool tc = is_tensor_core(algo);
   if (algo != MPM_NN_SIMT && !tc) return MPM_ERR_INVALID_ARG;
   if (tc && !bf16 && algo != MPM_NN_TCGEN05_PAIR) return MPM_ERR_UNSUPPORTED;
@@ -197,9 +196,11 @@ mpm_status nearest_neighbors_impl(const void* tokens, const int64_t* offsets, in
     return MPM_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const Workspace ws = carve(workspace, rows, batch, split_elems(rows, dim, dtype));
+  if (algo == MPM_NN_AUTO) algo = default_algo(dtype);
   st = run_affinity(tokens, offsets, batch, rows, dim, dtype, algo, chunk, ws, s);
   if (st != MPM_OK) return st;
-  return cuda_status(mpm::launch_decode_nn(batch, rows, ws, out_nn, out_score, num_sms(), s));
+  return cuda_status(mpm::launch_decode_nn(tokens, batch, rows, dim, chunk, for_algo(ws, algo, dtype), out_nn,
+                                           out_score, num_sms(), s));
 }
 
 mpm_status merge_impl(const void* tokens, const int64_t* offsets, int32_t batch, int64_t rows, int32_t dim,
@@ -253,7 +254,7 @@ mpm_status merge_impl(const void* tokens, const int64_t* offsets, int32_t batch,
   if (!mark(3) || !mark(4)) return MPM_ERR_CUDA;
   {
     const Range r("mpm.mutual_scan");
-    e = mpm::launch_mutual_compact(batch, rows, chunk, ws, out_map, out_offsets, sms, s);
+    e = mpm::launch_mutual_compact(tokens, batch, rows, dim, chunk, ws, out_map, out_offsets, sms, s);
   }
   if (e != cudaSuccess || !mark(5) || !mark(6)) return MPM_ERR_CUDA;
   {

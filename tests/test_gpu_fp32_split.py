@@ -107,3 +107,101 @@ def test_tiny_zero_and_non_finite_rows(mpm):
     s = oracle.cosine_affinity(x[good].astype(np.float64))
     chosen = s[np.arange(len(good)), np.searchsorted(good, nn[good])]
     np.testing.assert_allclose(score[good], chosen, rtol=0, atol=bound(96))
+
+
+def lone_features(counts, dim, power, seed):
+    """Images of normal tokens whose first two rows (where they have them) hold a feature of their own, 2^power."""
+    rng = np.random.default_rng(seed)
+    x = rng.standard_normal((sum(counts), dim))
+    x[:, :2] = 0.0
+    for a, n in zip(np.cumsum([0] + counts), counts):
+        for r in range(min(n, 2)):
+            x[a + r, r] = 2.0 ** power
+    return x.astype(np.float32), np.cumsum([0] + counts)
+
+
+@pytest.mark.parametrize("power", [12, 24, 44, 90])
+@pytest.mark.parametrize("dim,counts,chunk", [
+    (8, [40, 1, 0, 33], 0),
+    (12, [2, 2, 3], 0),
+    (196, [300, 2], 0),
+    (768, [129], 0),
+    (68, [700], 256),
+])
+def test_rows_with_a_huge_feature_of_their_own(mpm, dim, counts, chunk, power):
+    """Their cosines come from the small features alone, down to 2^-90 of the row's norm: the errors stay
+    relative to the terms that are added, as fp32's, and every row's neighbour is as good as the best.
+    (Cosines below fp32's range come back as 0.)"""
+    x, off = lone_features(counts, dim, power, seed=dim + power)
+    nn, score = mpm.nearest_neighbors(torch.from_numpy(x).to(DEV), torch.from_numpy(off).to(DEV), chunk=chunk)
+    nn, score = nn.cpu().numpy(), score.cpu().numpy()
+    for a, n in zip(off, counts):
+        run = chunk or max(n, 1)
+        for c0 in range(0, n, run):
+            img = x[a + c0:a + min(n, c0 + run)].astype(np.float64)
+            if len(img) == 1:
+                assert nn[a + c0] == -1
+                continue
+            s = oracle.cosine_affinity(img)
+            got = nn[a + c0:a + c0 + len(img)] - c0
+            chosen = s[np.arange(len(img)), got]
+            unit = img / np.linalg.norm(img, axis=1, keepdims=True)
+            terms = np.abs(unit) @ np.abs(unit).T      # what rounding errors are relative to
+            tol = bound(dim) * terms
+            error = np.abs(score[a + c0:a + c0 + len(img)] - chosen)
+            assert np.all(error <= tol[np.arange(len(img)), got] + 2.0 ** -148)
+            assert np.all(s - chosen[:, None] <= tol + tol[np.arange(len(img)), got][:, None])
+
+
+@pytest.mark.parametrize("dim,images,spare,chunk", [
+    (12, 1, 0, 0),         # one launch for the merge's tail
+    (196, 256, 0, 0),
+    (12, 300, 400, 0),     # its own launch before the scan
+    (100, 257, 300, 0),
+    (96, 3, 0, 256),       # the triples are the images' last chunks
+    (96, 5, 0, 256),
+])
+def test_merge_pairs_decided_by_small_features(mpm, dim, images, spare, chunk):
+    """Triples (-v, v, v + a feature of its own 2^44): the cosine of the last two is tiny, yet each is the other's
+    neighbour, so they are a pair in every image."""
+    rng = np.random.default_rng(dim + images)
+    head = chunk and 2 * rng.standard_normal((chunk, dim))
+    parts, counts = [], []
+    for _ in range(images):
+        v = rng.standard_normal(dim)
+        v[0] = 0.0
+        own = v.copy()
+        own[0] = 2.0 ** 44
+        img = np.stack([-v, v, own])
+        parts.append(np.concatenate([head, img]) if chunk else img)
+        counts.append(len(parts[-1]))
+    x = np.concatenate(parts).astype(np.float32)
+    off = torch.from_numpy(np.cumsum([0] + counts)).to(DEV)
+    xd = torch.cat([torch.from_numpy(x), torch.zeros(spare, dim)]).to(DEV)
+    ws = mpm.new_workspace(xd.shape[0], images, dim, xd.dtype, DEV)
+    for stage_events in ([None, True] if not chunk else [None]):
+        events = [torch.cuda.Event(enable_timing=True) for _ in range(8)] if stage_events else None
+        for e in events or []:
+            e.record()
+        out, out_off, rmap = mpm.merge(xd, off, workspace=ws, chunk=chunk, stage_events=events)
+        assert mpm.device_status(ws) == 0
+        rmap, out, out_off = rmap.cpu().numpy(), out.cpu().numpy(), out_off.cpu().numpy()
+        for b, (n, a) in enumerate(zip(counts, np.cumsum([0] + counts))):
+            local = rmap[a + n - 3:a + n]
+            assert local[2] == local[1] == local[0] + 1, b
+            assert out_off[b + 1] - out_off[b] == local[1] + 1
+            want = (x[a + n - 2] + x[a + n - 1]) * np.float32(0.5)
+            assert np.array_equal(out[out_off[b] + local[1]], want)
+
+
+def test_images_of_rows_with_huge_features_of_their_own(mpm):
+    """Every cosine lies below fp32's range (2^-200); the order of the small features' products still decides."""
+    rng = np.random.default_rng(12)
+    x = np.abs(rng.standard_normal((20, 32))) + 0.1
+    x[:, :20] = np.eye(20) * 2.0 ** 100
+    x = x.astype(np.float32)
+    nn, _ = mpm.nearest_neighbors(torch.from_numpy(x).to(DEV), torch.tensor([0, 20], device=DEV))
+    s = oracle.cosine_affinity(x.astype(np.float64))
+    best = np.sort(s, axis=1)
+    assert np.all(best[:, -1] > best[:, -2] * (1 + 2 * bound(32)))
+    assert np.array_equal(nn.cpu().numpy(), s.argmax(axis=1))
