@@ -286,6 +286,11 @@ __device__ __forceinline__ void mma_stage_full(uint32_t d_tmem, uint64_t a_desc,
 // 32 bytes), three fp16 products per slice, then the release commit.  The
 // stage's slices lie at a_desc (A high), +1024 (A low), +2048 (B high) and
 // +3072 (B low) in descriptor units of 16 bytes.
+// The eight products with a low part come before the four of high parts: the
+// accumulator is cut to fp32 at every addition, and small terms cost least
+// while the sum is small.  Against slice by slice, the rms error of the cosines
+// is 0.54 times as large at 64 features, 0.75 at 128, 0.96 at 768 (0.35 to 0.66
+// times that of three tf32 products), for the same time.
 __device__ __forceinline__ void mma_stage_split(uint32_t d_tmem, uint64_t a_desc, uint32_t idesc,
                                                  uint32_t accumulate, uint64_t* release) {
   asm volatile(
@@ -293,21 +298,25 @@ __device__ __forceinline__ void mma_stage_split(uint32_t d_tmem, uint64_t a_desc
       "setp.ne.b32 p, %3, 0;\n\t"
       "setp.ne.b32 q, %5, 0;\n\t"
       "add.s64 al, %1, 1024;\n\tadd.s64 bh, %1, 2048;\n\tadd.s64 bl, %1, 3072;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, bh, %2, p;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, bl, %2, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, bl, %2, p;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
       "add.s64 ah, %1, 2;\n\tadd.s64 al, %1, 1026;\n\tadd.s64 bh, %1, 2050;\n\tadd.s64 bl, %1, 3074;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bl, %2, q;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
       "add.s64 ah, %1, 4;\n\tadd.s64 al, %1, 1028;\n\tadd.s64 bh, %1, 2052;\n\tadd.s64 bl, %1, 3076;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bl, %2, q;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
       "add.s64 ah, %1, 6;\n\tadd.s64 al, %1, 1030;\n\tadd.s64 bh, %1, 2054;\n\tadd.s64 bl, %1, 3078;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bl, %2, q;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], al, bh, %2, q;\n\t"
+      "add.s64 bh, %1, 2048;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, bh, %2, q;\n\t"
+      "add.s64 ah, %1, 2;\n\tadd.s64 bh, %1, 2050;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
+      "add.s64 ah, %1, 4;\n\tadd.s64 bh, %1, 2052;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
+      "add.s64 ah, %1, 6;\n\tadd.s64 bh, %1, 2054;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], ah, bh, %2, q;\n\t"
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%4], %6;\n\t}"
       ::"r"(d_tmem), "l"(a_desc), "r"(idesc), "r"(accumulate), "r"(ptx::smem_addr(release)), "r"(1u),
       "h"(static_cast<uint16_t>(3))
@@ -340,14 +349,18 @@ __device__ __noinline__ void mma_partial_stage_bf16(uint32_t d_tmem, uint64_t a_
   }
   commit_both(release);
 }
+// The same order in a stage of fewer features.
 __device__ __noinline__ void mma_partial_stage_split(uint32_t d_tmem, uint64_t a_desc, uint32_t idesc, int kb,
                                                     int dim, uint64_t* release) {
   for (int kk = 0; kk < SPLIT_BK / 16 && kb * SPLIT_BK + kk * 16 < dim; ++kk) {
     const uint64_t ah = a_desc + 2 * kk, al = ah + (ATOM_BYTES >> 4);
     const uint64_t bh = ah + 2 * (ATOM_BYTES >> 4), bl = ah + 3 * (ATOM_BYTES >> 4);
-    mma_pair(d_tmem, ah, bh, idesc, (kb | kk) != 0 ? 1u : 0u);
-    mma_pair(d_tmem, ah, bl, idesc, 1u);
+    mma_pair(d_tmem, ah, bl, idesc, (kb | kk) != 0 ? 1u : 0u);
     mma_pair(d_tmem, al, bh, idesc, 1u);
+  }
+  for (int kk = 0; kk < SPLIT_BK / 16 && kb * SPLIT_BK + kk * 16 < dim; ++kk) {
+    const uint64_t ah = a_desc + 2 * kk;
+    mma_pair(d_tmem, ah, ah + 2 * (ATOM_BYTES >> 4), idesc, 1u);
   }
   commit_both(release);
 }
