@@ -27,36 +27,41 @@ __device__ __forceinline__ int64_t clamp64(int64_t v, int64_t lo, int64_t hi) {
 // -> 1.3 us).
 // ---------------------------------------------------------------------------
 // Sanitised offsets and work plan, by one block:
-//   soff[b] = min(rows, max_{b' <= b} max(off[b'], 0)), non-decreasing and in
-//             range whatever the caller passed (violations are reported);
+//   soff[b] = min(used, max_{b' <= b} max(off[b'], 0)) with used = off[batch]
+//             clamped to the rows there are: non-decreasing, in range and
+//             within the rows that prep covers, whatever the caller passed
+//             (violations are reported);
 //   plan[b] = number of affinity tiles of the images before b.
 __device__ __forceinline__ void write_plan(const int64_t* __restrict__ offsets, int batch, int64_t rows,
                                            const AffinityTile& tile, const Workspace& ws) {
   __shared__ int64_t sh[32];
   __shared__ int64_t ends[kThreads + 1];
   __shared__ int bad;
-  int64_t off0 = 0;
   if (threadIdx.x == 0) {
     ws.status[0] = 0;
     ws.status[1] = 0;
     ws.status[2] = 0;
-    off0 = offsets[0];
-    bad = off0 != 0 ? 0 : -1;
-    ends[0] = clamp64(off0, 0, rows);
-    ws.soff[0] = ends[0];
+    bad = -1;
   }
   __syncthreads();
+  const int64_t used = clamp64(offsets[batch], 0, rows);
   int64_t acc = 0;
   for (int base = 0; base < batch; base += kThreads) {
     // Image `idx`: from soff[idx], which the thread before has, to soff[idx + 1].
     const int idx = base + threadIdx.x;
     int64_t end = 0;
     if (idx < batch) {
-      const int64_t raw = offsets[idx + 1];
-      if (raw < offsets[idx] || raw > rows) atomicCAS(&bad, -1, idx + 1);
-      end = clamp64(raw, 0, rows);
+      const int64_t raw = offsets[idx + 1], prev = offsets[idx];
+      if (raw < prev || raw > rows) atomicCAS(&bad, -1, idx + 1);
+      end = clamp64(raw, 0, used);
+      if (idx == 0) {
+        if (prev != 0) atomicExch(&bad, 0);
+        const int64_t first = clamp64(prev, 0, used);
+        ends[0] = ws.soff[0] = first;
+        end = end > first ? end : first;
+      }
     }
-    const int64_t carry = ends[0];
+    const int64_t carry = base > 0 ? ends[0] : 0;
     int64_t last;
     end = block_incl_max<int64_t>(end, sh, &last, 0);
     end = end > carry ? end : carry;

@@ -91,3 +91,25 @@ def test_bad_offsets(mpm, bad):
     one, two = both_paths(mpm, x, torch.tensor(bad, dtype=torch.int64, device=DEV))
     assert_same(one, two)
     assert one[3] == 6
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("bad", [[0, 150, 100], [0, 150, 40, 100], [0, 100, -3], [0, 1 << 40, 149]])
+def test_results_do_not_depend_on_the_workspace_when_the_last_offset_is_not_the_largest(mpm, bad, dtype):
+    """Rows from the last offset on belong to no image: nothing is computed from what the workspace held for them."""
+    gen = torch.Generator(device=DEV).manual_seed(4)
+    off = torch.tensor(bad, dtype=torch.int64, device=DEV)
+    for rows in (150, 1200):
+        x = torch.randn(rows, 64, generator=gen, device=DEV).to(dtype)
+        results = []
+        for fill in (0x00, 0x5A, 0xFF):
+            ws = mpm.new_workspace(rows, len(bad) - 1, 64, dtype, DEV)
+            ws.fill_(fill)
+            out = torch.full_like(x, 7.0)
+            rmap = torch.full((rows,), -5, dtype=torch.int32, device=DEV)
+            _, out_off, _ = mpm.merge(x, off, workspace=ws, out_tokens=out, out_map=rmap)
+            results.append((out, out_off, rmap, mpm.device_status(ws)))
+            assert torch.all(rmap[max(bad[-1], 0):] == -5)
+            assert results[-1][3] == 6
+        for one in results[1:]:
+            assert_same(results[0], one)
