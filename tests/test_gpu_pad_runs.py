@@ -1,4 +1,4 @@
-"""Pad and unpad where their split into runs of rows can go wrong:
+"""Pad and unpad where their split into rows or runs of rows can go wrong:
 padded lengths below, at and just past a run, the shortest and longest rows,
 odd vector counts, empty images, many images, and images longer than the
 padded length.  Both are copies, so everything is bit-exact."""
@@ -34,9 +34,16 @@ def mpm():
     (torch.bfloat16, 64, [3] * 5000, 3),                # many short images
     (torch.bfloat16, 16, [2000, 1500, 0, 1999] * 40, 2001),   # several rounds of the whole GPU
     (torch.bfloat16, 72, [30, 90, 10], 41),             # one image is cut
-    (torch.bfloat16, 64, [900] * 200, 900),             # runs of 22 rows
-    (torch.bfloat16, 1024, [65, 700, 0] * 30, 701),     # 128 vectors: runs of 3 rows
-    (torch.float32, 516, [300, 299] * 40, 300),         # 129 vectors: no good fill
+    (torch.bfloat16, 64, [900] * 200, 900),             # runs of 24 rows
+    (torch.bfloat16, 1024, [65, 700, 0] * 30, 701),     # 128 vectors, the most with four in flight
+    (torch.float32, 516, [300, 299] * 40, 300),         # 129 vectors
+    # Either side of the rule that chooses between runs and a row a warp.
+    (torch.bfloat16, 384, [300, 290] * 10, 301),        # 48 vectors, more rows than warps: runs
+    (torch.bfloat16, 384, [50, 0, 49], 50),             # fewer: a row a warp
+    (torch.bfloat16, 392, [300, 290] * 10, 301),        # 49 vectors, few rows a warp: a row a warp
+    (torch.bfloat16, 768, [150, 120] * 85, 151),        # 96 vectors, many: runs
+    (torch.bfloat16, 776, [150, 120] * 85, 151),        # 97: a row a warp, four vectors in flight
+    (torch.bfloat16, 1032, [40] + [0, 33] * 20, 36),     # 129: six in flight; one image is cut
 ])
 def test_runs(mpm, dtype, dim, counts, max_len):
     gen = torch.Generator(device=DEV).manual_seed(8)
