@@ -238,9 +238,11 @@ __device__ __noinline__ RowScale odd_row_scale(const uint4* src, int nvec, float
   return {s1, s2, scalbnf(inv, -up)};
 }
 
+// May the scale of a row be taken from its sum of squares?
+__device__ __forceinline__ bool ordinary_sumsq(float sumsq) { return sumsq >= 0x1p-100f && sumsq <= 0x1p100f; }
 // Scale of a row from its sum of squares `sumsq` (the same in every lane).
 __device__ __forceinline__ RowScale row_scale(const uint4* src, int nvec, float sumsq) {
-  if (!(sumsq >= 0x1p-100f && sumsq <= 0x1p100f)) return odd_row_scale(src, nvec, sumsq);
+  if (!ordinary_sumsq(sumsq)) return odd_row_scale(src, nvec, sumsq);
   const float norm = sqrtf(sumsq);
   const int e = 14 - (static_cast<int>(__float_as_uint(norm) >> 23) - 127);
   return {__uint_as_float(static_cast<uint32_t>(127 + e) << 23), 1.0f,
@@ -309,92 +311,139 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
 
 // ---------------------------------------------------------------------------
 // fp32 rows that the fp16 parts cannot decide.  An element's parts are off by
-// at most 2^-39 of its row's norm (above), so a cosine by at most about 2^-38
-// sqrt(D).  That is no more than fp32's own rounding as long as the cosine is
-// above 2^-15 sqrt(D) in size.  A row whose best cosine is smaller (rows with
-// a huge feature of their own: its other features decide, and may have lost
-// bits or vanished) has its neighbour found again by fp32 products of its
-// run's tokens.  The kernels that read the keys of an fp32 call do that
-// first.  Ordinary tokens never come here: the best of 1000 random cosines is
-// about 3 / sqrt(D).  The check costs 0.2 us in the one-launch tail (one image
-// of 1024 x 192: 12.8 -> 13.0) and 0.2 to 1.1 in the scan (64 x 1024 x 192:
-// 80.5 -> 81.3; 256 x 256 x 32: 45.0 -> 46.1).  A kernel of its own before the
-// scan cost 1.6 to 2.4.
+// at most 2^-39 of its row's norm (above): a cosine by about 2^-39 as the
+// errors' signs go, by 2^-39 sqrt(D) at worst.  A cosine of 2^-15 or more is
+// right to 2^-24, at worst 2^-24 sqrt(D), of its size, less than the products'
+// sum loses.  A row whose best cosine is smaller (rows with a huge feature of
+// their own: its other features decide, and may have lost bits or vanished)
+// has its neighbour found again by fp32 products of its run's tokens.  The
+// kernels that read the keys of an fp32 call do that first.  Ordinary tokens
+// hardly ever come here: the best of 1000 random cosines is about 3 / sqrt(D).
+//
+// The check reads nothing that the kernels do not read anyway and costs 0.1 to
+// 0.5 us a merge (1024 x 192: 12.8 -> 13.0 us, 64 x 1024 x 192 80.9 -> 81.2, 64 x
+// 1024 x 384 117.0 -> 117.3); a kernel of its own before the scan cost 1.6 to 2.4.
+// Finding a row again takes one block: 0.12 ms among 1024 x 192, 0.19 ms among
+// 4096 x 768, and as long again for each further such row.
 // ---------------------------------------------------------------------------
-// Is the row's best cosine too small to trust?  Zero rows (all their cosines
-// are exactly 0) have the largest inverse norm, 1e12; every other row's, scaled,
-// is at most 2^-7 or so.
-// `limit` is 2^-15 sqrt(D).
-__device__ __forceinline__ bool undecided(unsigned long long key, float inv_norm, float limit) {
-  return (key != 0ull) & (inv_norm < 1e11f) & (fabsf(key_score(key) * inv_norm) < limit);
+// Is the row's best cosine too small to trust?  Its score is the cosine times
+// the scaled row's norm, 2^14 to 2^15: above 1 it needs no look at the norm.
+// Zero rows, whose cosines are exactly 0, need nothing: their inverse norm is
+// 1e12, every other row's, scaled, at most 2^-7 or so.
+__device__ __forceinline__ bool maybe_undecided(unsigned long long key) {
+  return (key != 0ull) & (fabsf(key_score(key)) < 1.0f);
 }
-float decide_limit(int dim) { return 0x1p-15f * sqrtf(static_cast<float>(dim)); }
+__device__ __forceinline__ bool undecided(unsigned long long key, float inv_norm) {
+  return (key != 0ull) & (inv_norm < 1e11f) & (fabsf(key_score(key) * inv_norm) < 0x1p-15f);
+}
 
-// The best neighbour's packed key of row `row`, whose image starts at `base`,
-// among the n rows from base + first on.  Scores as the affinity kernel's:
-// products of the scaled rows times the neighbour's scaled inverse norm; ties
-// to the lowest index, NaN never wins.  Scores are compared 2^96 times as
-// large (at most 2^126), so that products of two rows' smallest features do
-// not vanish.  By a whole warp.
-__device__ __noinline__ unsigned long long exact_key(const float* tokens, int dim, int64_t base, int first, int n,
-                                                     int64_t row) {
+// Does any of the rows r0 .. r1 - 1 have an element that its parts do not hold to
+// 22 bits (below 2^-17 of the norm, but not 0)?  If none has, small cosines are
+// right as they are, those of one-hot rows for instance.  By a whole block.
+__device__ __noinline__ bool any_cut_element(const float* __restrict__ tokens, int dim, int64_t r0, int64_t r1) {
+  const int lane = threadIdx.x & 31, nvec = dim >> 2;
+  const int64_t warps = blockDim.x >> 5;
+  for (int64_t w0 = r0; w0 < r1; w0 += 8 * warps) {
+    bool cut = false;
+    const int64_t end = w0 + 8 * warps < r1 ? w0 + 8 * warps : r1;
+    for (int64_t r = w0 + (threadIdx.x >> 5); r < end; r += warps) {
+      const uint4* const x = reinterpret_cast<const uint4*>(tokens) + r * nvec;
+      float s = 0.f, least = INFINITY;
+#pragma unroll 2
+      for (int v = lane; v < nvec; v += 32) {
+        const uint4 q = __ldg(x + v);
+        const float* f = reinterpret_cast<const float*>(&q);
+        s += sumsq16(q, false);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) least = f[k] == 0.f ? least : fminf(least, fabsf(f[k]));
+      }
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) {
+        s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+        least = fminf(least, __shfl_xor_sync(0xFFFFFFFFu, least, d));
+      }
+      cut |= least < INFINITY && !(ordinary_sumsq(s) && least >= 0x1p-17f * sqrtf(s));
+    }
+    if (__syncthreads_or(cut)) return true;
+  }
+  return false;
+}
+
+// `key`, or the packed row's key found again where `redo` is set: the best of
+// its run by the affinity kernel's scores, products of the scaled rows times
+// the neighbour's scaled inverse norm.  Ties go to the lowest index and NaN
+// never wins.  Scores are compared 2^96 times as large (at most 2^126), so that
+// products of two rows' smallest features do not vanish.  Called by all threads
+// of a block: one row at a time, its candidates dealt over the warps.
+__device__ __noinline__ unsigned long long decide(bool redo, unsigned long long key, int64_t row,
+                                                  const float* __restrict__ tokens, int dim, int batch, int chunk,
+                                                  const int64_t* soff) {
+  __shared__ unsigned long long turn, best;  // the next row (and its thread below it); its best key
   const int lane = threadIdx.x & 31, nvec = dim >> 2;
   const auto sum = [](float s) {
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
     return s;
   };
-  const auto scale_of = [&](const uint4* x) {
-    float s = 0.f;
-#pragma unroll 1
-    for (int v = lane; v < nvec; v += 32) s += sumsq16(__ldg(x + v), false);
-    return row_scale(x, nvec, sum(s));
-  };
-  const uint4* const rows = reinterpret_cast<const uint4*>(tokens);
-  const uint4* const x = rows + row * nvec;
-  const RowScale a = scale_of(x);
-  float best = -INFINITY;
-  int at = -1;
-  for (int j = first; j < first + n; ++j) {
-    if (base + j == row) continue;
-    const uint4* const y = rows + (base + j) * nvec;
-    const RowScale b = scale_of(y);
-    float dot = 0.f;
-#pragma unroll 1
+  // Sums of y's squares and of its products with x, each value times s1 s2.
+  const auto products = [&](const uint4* x, const uint4* y, float xs1, float xs2, float ys1, float ys2) {
+    float2 r = make_float2(0.f, 0.f);
+#pragma unroll 2
     for (int v = lane; v < nvec; v += 32) {
       const uint4 p = __ldg(x + v), q = __ldg(y + v);
       const float* f = reinterpret_cast<const float*>(&p);
       const float* g = reinterpret_cast<const float*>(&q);
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        dot = fmaf(f[k] * a.s1 * a.s2 * 0x1p48f, g[k] * b.s1 * b.s2 * 0x1p48f, dot);
+      for (int k = 0; k < 4; ++k) {
+        const float w = g[k] * ys1 * ys2;
+        r.x = fmaf(w, w, r.x);
+        r.y = fmaf(f[k] * xs1 * xs2, w, r.y);
+      }
     }
-    const float score = sum(dot) * b.inv;
-    if (score > best) {
-      best = score;
-      at = j;
+    return make_float2(sum(r.x), sum(r.y));
+  };
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      turn = ~0ull;
+      best = 0ull;
     }
-  }
-  return at < 0 ? 0ull : make_key(best * 0x1p-96f, at);
-}
-
-// `key`, or the row's key found again where `redo` is set.  Called by whole
-// warps, with the packed row of each lane.
-__device__ __noinline__ unsigned long long decide(bool redo, unsigned long long key, int64_t row, const float* tokens,
-                                                  int dim, int batch, int chunk, const int64_t* soff) {
-  const int lane = threadIdx.x & 31;
-  for (uint32_t left = __ballot_sync(0xFFFFFFFFu, redo); left != 0u; left &= left - 1u) {
-    const int src = __ffs(static_cast<int>(left)) - 1;
-    const int64_t r = __shfl_sync(0xFFFFFFFFu, row, src);
+    __syncthreads();
+    const unsigned long long mine = static_cast<unsigned long long>(row) << 10 | threadIdx.x;
+    if (redo) atomicMin(&turn, mine);
+    __syncthreads();
+    const unsigned long long now = turn;
+    if (now == ~0ull) return key;
+    const int64_t r = static_cast<int64_t>(now >> 10);
     const int b = find_image(soff, batch, r);
     const int64_t base = soff[b];
     const int n = static_cast<int>(soff[b + 1] - base), local = static_cast<int>(r - base);
     const int first = chunk > 0 ? (local / chunk) * chunk : 0;
-    const int len = chunk > 0 && n - first > chunk ? chunk : n - first;
-    const unsigned long long k = exact_key(tokens, dim, base, first, len, r);
-    if (lane == src) key = k;
+    const int end = chunk > 0 && n - first > chunk ? first + chunk : n;
+    const uint4* const rows = reinterpret_cast<const uint4*>(tokens);
+    const uint4* const x = rows + r * nvec;
+    const RowScale a = row_scale(x, nvec, products(x, x, 1.f, 1.f, 1.f, 1.f).x);
+    unsigned long long top = 0ull;
+    for (int j = first + static_cast<int>(threadIdx.x >> 5); j < end; j += static_cast<int>(blockDim.x >> 5)) {
+      if (j == local) continue;
+      const uint4* const y = rows + (base + j) * nvec;
+      float2 p = products(x, y, a.s1 * 0x1p24f, a.s2 * 0x1p24f, 1.f, 1.f);
+      float score = p.y * (0x1p48f / fmaxf(sqrtf(p.x), 1e-12f));
+      if (!ordinary_sumsq(p.x)) {
+        const RowScale c = odd_row_scale(y, nvec, p.x);
+        p = products(x, y, a.s1 * 0x1p24f, a.s2 * 0x1p24f, c.s1, c.s2);
+        score = p.y * (c.inv * 0x1p48f);
+      }
+      const unsigned long long k = score == score ? make_key(score, j) : 0ull;
+      top = k > top ? k : top;
+    }
+    if (lane == 0 && top != 0ull) atomicMax(&best, top);
+    __syncthreads();
+    if (redo && mine == now) {
+      key = best == 0ull ? 0ull : make_key(key_score(best) * 0x1p-96f, key_index(best));
+      redo = false;
+    }
   }
-  return key;
 }
 
 // ---------------------------------------------------------------------------
@@ -416,6 +465,7 @@ __device__ __noinline__ unsigned long long decide(bool redo, unsigned long long 
 constexpr int kScanThreads = 1024;
 constexpr int kScanElems = 4;
 constexpr int kScanMaxCluster = 8;
+constexpr int kAgain = 1 << 30;  // in a block's count: its image has to be scanned again
 // Images whose counts every block of the pair average adds up itself.
 constexpr int kStagedImages = 1024;
 
@@ -443,13 +493,57 @@ __device__ __forceinline__ void store_to_rank(int32_t* p, uint32_t rank, int32_t
   asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
 }
 
-// SPLIT: fp32 tokens, whose keys (a row's and its neighbour's) decide() checks
-// first.
+// May row i of an image of n rows have neighbour j?  b(i) lies in i's chunk (the
+// whole image without chunking), and only a token alone in its chunk has none.
+__device__ __forceinline__ bool neighbour_ok(int j, int i, int n, int chunk) {
+  const int cstart = chunk > 0 ? (i / chunk) * chunk : 0;
+  const int clen = chunk > 0 ? (n - cstart < chunk ? n - cstart : chunk) : n;
+  return j < 0 ? clen == 1 : j < n && j != i && j >= cstart && j - cstart < clen;
+}
+
+// One image's scan once more, by a whole block, with undecided keys found again;
+// returns the number of representatives.
+__device__ __noinline__ int scan_again(const float* tokens, int batch, int dim, int chunk, const int64_t* soff,
+                                       const unsigned long long* keys, const float* inv_norm, int b, int32_t* out_map,
+                                       int2* out_reps) {
+  __shared__ int32_t sh[32];
+  const int64_t base = soff[b];
+  const int n = static_cast<int>(soff[b + 1] - base);
+  const bool cut = any_cut_element(tokens, dim, base, base + n);
+  int carry = 0;
+  for (int c0 = 0; c0 < n; c0 += static_cast<int>(blockDim.x)) {
+    const int i = c0 + static_cast<int>(threadIdx.x);
+    const bool live = i < n;
+    unsigned long long key = live ? keys[base + i] : 0ull;
+    key = decide(cut && live && undecided(key, inv_norm[base + i]), key, base + i, tokens, dim, batch, chunk, soff);
+    int j = key_index(key);
+    if (!live || !neighbour_ok(j, i, n, chunk)) j = -1;
+    key = j >= 0 ? keys[base + j] : 0ull;
+    key = decide(cut && j >= 0 && undecided(key, inv_norm[base + j]), key, base + j, tokens, dim, batch, chunk, soff);
+    if (key_index(key) != i) j = -1;
+    const bool rep = live && (j < 0 || i < j);
+    int total;
+    const int incl = block_incl_sum<int>(rep ? 1 : 0, sh, &total);
+    if (rep) {
+      const int r = carry + incl - 1;
+      out_map[base + i] = r;
+      if (j >= 0) out_map[base + j] = r;
+      out_reps[base + r] = make_int2(i, j);
+    }
+    carry += total;
+  }
+  return carry;
+}
+
+// SPLIT: fp32 tokens.  An image with an undecided key is left to its first
+// block, which scans it again from the start: a call in the middle of the loop
+// cost every fp32 merge 1 to 6 us in spilled registers or blocks an SM.  (One
+// block an SM only where the registers of four rows a thread and a cluster ask
+// for it.)
 template <int ELEMS, bool CLUSTER, bool SPLIT>
-__global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(const float* __restrict__ tokens, int batch,
-                                                                      int dim, int chunk, float limit, Workspace ws,
-                                                                      int32_t* __restrict__ out_map,
-                                                                      int64_t* __restrict__ out_offsets) {
+__global__ void __launch_bounds__(kScanThreads, CLUSTER && ELEMS > 1 ? 1 : 2)
+    mutual_compact_kernel(const float* __restrict__ tokens, int batch, int dim, int chunk, Workspace ws,
+                          int32_t* __restrict__ out_map, int64_t* __restrict__ out_offsets) {
   MPM_TRACE_BEGIN(MPM_TRACE_MUTUAL);
   // Every block of the cluster runs before any stores into another's memory.
   if (CLUSTER) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -469,53 +563,47 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(const floa
   const int n = static_cast<int>(ws.soff[b + 1] - base);
   const int round_rows = blocks * kScanThreads;  // rows of one element per thread
   int carry = 0, buf = 0;
+  [[maybe_unused]] bool again = false;
   for (int64_t c0 = 0; c0 < n; c0 += static_cast<int64_t>(round_rows) * ELEMS, buf ^= 1) {
     const int left = n - static_cast<int>(c0);
     const int elems = left >= round_rows * ELEMS ? ELEMS : (left + round_rows - 1) / round_rows;
     const int64_t first = c0 + rank * elems * kScanThreads + static_cast<int>(threadIdx.x);
     int j[ELEMS];
     uint32_t reps[ELEMS];  // ballot of the warp's representatives
+    [[maybe_unused]] bool redo = false;
 #pragma unroll
     for (int e = 0; e < ELEMS; ++e) {
       const int64_t i = first + e * kScanThreads;
-      const bool live = e < elems && i < n;
-      unsigned long long key = live ? ws.keys[base + i] : 0ull;
-      if constexpr (SPLIT) {
-        const float inv = live ? ws.inv_norm[base + i] : 0.f;
-        const bool redo = undecided(key, inv, limit);
-        if (__any_sync(0xFFFFFFFFu, redo)) key = decide(redo, key, base + i, tokens, dim, batch, chunk, ws.soff);
-      }
+      const unsigned long long key = (e < elems && i < n) ? ws.keys[base + i] : 0ull;
+      if (SPLIT) redo |= maybe_undecided(key);
       j[e] = key_index(key);
     }
 #pragma unroll
     for (int e = 0; e < ELEMS; ++e) {
       const int i = static_cast<int>(first + e * kScanThreads);  // used only where the row exists
+      bool rep = false;
       if (e < elems && first + e * kScanThreads < n) {
-        // b(i) lies in i's chunk (the whole image without chunking), and only a
-        // token alone in its chunk has none.
-        const int cstart = chunk > 0 ? (i / chunk) * chunk : 0;
-        const int clen = chunk > 0 ? (n - cstart < chunk ? n - cstart : chunk) : n;
-        if (j[e] >= n || j[e] == i || (j[e] < 0 && clen > 1) ||
-            (j[e] >= 0 && (j[e] < cstart || j[e] - cstart >= clen))) {
+        if (!neighbour_ok(j[e], i, n, chunk)) {
           report(ws.status, MPM_ERR_DEVICE_CHECK, static_cast<int32_t>(base + i));
           j[e] = -1;
         }
+        // (i, j) is a pair of P when b(j) = i as well (Section 3.2).
+        if (j[e] >= 0) {
+          const unsigned long long key = ws.keys[base + j[e]];
+          if (SPLIT) redo |= maybe_undecided(key);
+          if (key_index(key) != i) j[e] = -1;
+        }
+        rep = j[e] < 0 || i < j[e];
       }
-      // (i, j) is a pair of P when b(j) = i as well (Section 3.2).
-      if constexpr (SPLIT) {
-        unsigned long long key = j[e] >= 0 ? ws.keys[base + j[e]] : 0ull;
-        const float inv = j[e] >= 0 ? ws.inv_norm[base + j[e]] : 0.f;
-        const bool redo = undecided(key, inv, limit);
-        if (__any_sync(0xFFFFFFFFu, redo)) key = decide(redo, key, base + j[e], tokens, dim, batch, chunk, ws.soff);
-        if (key_index(key) != i) j[e] = -1;
-      } else {
-        if (j[e] >= 0 && key_index(ws.keys[base + j[e]]) != i) j[e] = -1;
-      }
-      const bool rep = e < elems && first + e * kScanThreads < n && (j[e] < 0 || i < j[e]);
       reps[e] = __ballot_sync(0xFFFFFFFFu, rep);
       if (lane == 0) warp_count[buf][e][warp] = __popc(reps[e]);
     }
-    __syncthreads();
+    if constexpr (SPLIT) {
+      again = __syncthreads_or(redo) != 0;
+      if (!CLUSTER && again) break;
+    } else {
+      __syncthreads();
+    }
     // Representatives of this block's run before each of this warp's elements.
     int start[ELEMS], total = 0;
 #pragma unroll
@@ -531,14 +619,19 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(const floa
     if constexpr (CLUSTER) {
       // The other blocks reach this round's barrier only after they read the
       // counts of the round before the last, which this buffer held.
+      if (SPLIT && again) total |= kAgain;
       if (threadIdx.x < static_cast<unsigned>(blocks)) store_to_rank(&block_count[buf][rank], threadIdx.x, total);
       __syncwarp();
       asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+      if (SPLIT) again = false;
       for (int r = 0; r < blocks; ++r) {
-        const int t = block_count[buf][r];
+        int t = block_count[buf][r];
+        if (SPLIT) again |= t >= kAgain;
+        if (SPLIT) t &= kAgain - 1;
         run_base += r < rank ? t : 0;
         carry += t;
       }
+      if (SPLIT && again) break;
     } else {
       carry += total;
     }
@@ -554,6 +647,8 @@ __global__ void __launch_bounds__(kScanThreads) mutual_compact_kernel(const floa
     }
   }
   if (rank != 0) return;
+  if (SPLIT && again)
+    carry = scan_again(tokens, batch, dim, chunk, ws.soff, ws.keys, ws.inv_norm, b, out_map, ws.reps);
   if (threadIdx.x == 0) ws.count[b] = carry;
   if (batch <= kStagedImages) return;
   // More images than the pair average's blocks turn into offsets themselves:
@@ -737,8 +832,8 @@ __device__ __forceinline__ void average_row(const uint8_t* __restrict__ tokens, 
 template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __restrict__ tokens,
                                                               uint8_t* __restrict__ out, int batch, int rows,
-                                                              int chunk, int row_bytes, bool bf16, float limit,
-                                                              Workspace ws, int32_t* __restrict__ out_map,
+                                                              int chunk, int row_bytes, bool bf16, Workspace ws,
+                                                              int32_t* __restrict__ out_map,
                                                               int64_t* __restrict__ out_offsets) {
   __shared__ int32_t first_s[kTailImages + 1];   // first input row of every image
   __shared__ int32_t start_s[kTailImages + 1];   // first output row of every image
@@ -752,31 +847,25 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
   const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
   int j[kTailElems], image[kTailElems];
   [[maybe_unused]] bool redo = false;
-  {
-    unsigned long long key[kTailElems];
-    [[maybe_unused]] float inv[kTailElems];
 #pragma unroll
-    for (int e = 0; e < kTailElems; ++e) {
-      const int i = e * kThreads + tid;
-      key[e] = i < rows ? ws.keys[i] : 0ull;
-      if (SPLIT) inv[e] = i < rows ? ws.inv_norm[i] : 0.f;
-    }
-#pragma unroll
-    for (int e = 0; e < kTailElems; ++e) {
-      j[e] = key_index(key[e]);
-      if (SPLIT) redo |= undecided(key[e], inv[e], limit);
-    }
+  for (int e = 0; e < kTailElems; ++e) {
+    const int i = e * kThreads + tid;
+    const unsigned long long key = i < rows ? ws.keys[i] : 0ull;
+    if (SPLIT) redo |= maybe_undecided(key);
+    j[e] = key_index(key);
   }
   for (int idx = tid; idx <= batch; idx += kThreads) first_s[idx] = static_cast<int32_t>(ws.soff[idx]);
-  __syncthreads();
+  bool some = false;
+  if (SPLIT) some = __syncthreads_or(redo); else __syncthreads();
   const int lead = first_s[0], used = first_s[batch];  // rows before the first image belong to none
-  if (SPLIT && __any_sync(0xFFFFFFFFu, redo)) {
-    // Rare: every block finds these rows' neighbours again for itself.
+  if (SPLIT && some) {
+    if (blockIdx.x != 0) return;  // rare: one block does it all, so that none repeats the search
+    const bool cut = any_cut_element(reinterpret_cast<const float*>(tokens), row_bytes >> 2, lead, used);
     for (int e = 0; e < kTailElems; ++e) {
       const int i = e * kThreads + tid;
       const bool live = i >= lead && i < used;
       const unsigned long long key = live ? ws.keys[i] : 0ull;
-      const int again = key_index(decide(live && undecided(key, ws.inv_norm[i], limit), key, i,
+      const int again = key_index(decide(cut && live && undecided(key, ws.inv_norm[i]), key, i,
                                          reinterpret_cast<const float*>(tokens), row_bytes >> 2, batch, chunk, ws.soff));
 #pragma unroll
       for (int k = 0; k < kTailElems; ++k) j[k] = k == e && live ? again : j[k];
@@ -794,11 +883,7 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
     const int base = first_s[b], n = first_s[b + 1] - base, local = i - base;
     int nn = -1;
     if (i >= lead && i < used) {
-      // As in mutual_compact_kernel.
-      const int cstart = chunk > 0 ? (local / chunk) * chunk : 0;
-      const int clen = chunk > 0 ? (n - cstart < chunk ? n - cstart : chunk) : n;
-      if (j[e] >= n || j[e] == local || (j[e] < 0 && clen > 1) ||
-          (j[e] >= 0 && (j[e] < cstart || j[e] - cstart >= clen))) {
+      if (!neighbour_ok(j[e], local, n, chunk)) {
         if (blockIdx.x == 0) report(ws.status, MPM_ERR_DEVICE_CHECK, i);
       } else if (j[e] >= 0) {
         nn = base + j[e];
@@ -832,8 +917,9 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
     }
   }
   __syncthreads();
-  const int64_t nwarps = static_cast<int64_t>(gridDim.x) * (kThreads / 32);
-  for (int64_t t = warp_number(blockIdx.x, gridDim.x, true); t < total; t += nwarps) {
+  const int blocks = some ? 1 : static_cast<int>(gridDim.x);
+  const int64_t nwarps = static_cast<int64_t>(blocks) * (kThreads / 32);
+  for (int64_t t = warp_number(blockIdx.x, blocks, true); t < total; t += nwarps) {
     const uint32_t r = list_s[t];
     const int first = static_cast<int>(r & 0xFFFFu), second = static_cast<int>(r >> 16);
     const bool pair = second != 0xFFFF;
@@ -860,18 +946,21 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
 // ---------------------------------------------------------------------------
 template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 4) decode_nn_kernel(const float* __restrict__ tokens, int batch, int dim,
-                                                                int chunk, float limit, Workspace ws,
-                                                                int32_t* __restrict__ nn, float* __restrict__ score) {
+                                                                int chunk, Workspace ws, int32_t* __restrict__ nn,
+                                                                float* __restrict__ score) {
   wait_for_previous_grid();
   const int64_t used = ws.soff[batch];
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t w0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + (threadIdx.x & ~31u); w0 < used; w0 += stride) {
-    const int64_t g = w0 + (threadIdx.x & 31);
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
+  for (int64_t b0 = static_cast<int64_t>(blockIdx.x) * kThreads; b0 < used; b0 += stride) {
+    const int64_t g = b0 + threadIdx.x;
     unsigned long long k = g < used ? ws.keys[g] : 0ull;
     const float inv = g < used ? ws.inv_norm[g] : 0.f;
-    if (SPLIT) {
-      const bool redo = undecided(k, inv, limit);
-      if (__any_sync(0xFFFFFFFFu, redo)) k = decide(redo, k, g, tokens, dim, batch, chunk, ws.soff);
+    if (SPLIT && __syncthreads_or(maybe_undecided(k))) {
+      // The rows of all images that this block's rows belong to.
+      const int64_t last = b0 + kThreads < used ? b0 + kThreads - 1 : used - 1;
+      const int64_t r0 = ws.soff[find_image(ws.soff, batch, b0)], r1 = ws.soff[find_image(ws.soff, batch, last) + 1];
+      if (any_cut_element(tokens, dim, r0, r1))
+        k = decide(undecided(k, inv), k, g, tokens, dim, batch, chunk, ws.soff);
     }
     if (g >= used) continue;
     nn[g] = key_index(k);
@@ -1158,8 +1247,8 @@ cudaError_t launch_mutual_compact(const void* tokens, int batch, int64_t rows, i
                       : (more ? mutual_compact_kernel<kScanElems, false, S> : mutual_compact_kernel<1, false, S>);
   };
   const auto kernel = ws.split_hi != nullptr ? pick(std::true_type{}) : pick(std::false_type{});
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<const float*>(tokens), batch, dim, chunk32, decide_limit(dim), ws,
-                            out_map, out_offsets);
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<const float*>(tokens), batch, dim, chunk32, ws, out_map,
+                            out_offsets);
 }
 
 cudaError_t launch_pair_average(const void* tokens, void* out_tokens, int batch, int64_t rows,
@@ -1212,7 +1301,7 @@ cudaError_t launch_merge_tail(const void* tokens, void* out_tokens, int batch, i
     return launch_dependent(kernel, dim3(row_grid(rows, grid_for(num_sms, per_sm)).blocks), dim3(kThreads), 0, stream,
                             static_cast<const uint8_t*>(tokens), static_cast<uint8_t*>(out_tokens), batch,
                             static_cast<int>(rows), chunk < rows ? static_cast<int>(chunk) : 0,
-                            dim * (bf16 ? 2 : 4), bf16, decide_limit(dim), ws, out_map, out_offsets);
+                            dim * (bf16 ? 2 : 4), bf16, ws, out_map, out_offsets);
   };
   if (ws.split_hi != nullptr) {
     static const int per_sm = resident_per_sm(merge_tail_kernel<true>, kThreads, 8);
@@ -1227,7 +1316,7 @@ cudaError_t launch_decode_nn(const void* tokens, int batch, int64_t rows, int di
   const auto launch = [&](auto kernel) {
     return launch_dependent(kernel, dim3(grid_for(num_sms, 4)), dim3(kThreads), 0, stream,
                             static_cast<const float*>(tokens), batch, dim,
-                            chunk < rows ? static_cast<int>(chunk) : 0, decide_limit(dim), ws, out_nn, out_score);
+                            chunk < rows ? static_cast<int>(chunk) : 0, ws, out_nn, out_score);
   };
   return ws.split_hi != nullptr ? launch(decode_nn_kernel<true>) : launch(decode_nn_kernel<false>);
 }

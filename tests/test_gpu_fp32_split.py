@@ -223,3 +223,16 @@ def test_error_is_no_larger_than_that_of_three_tf32_products(mpm, dim, rms):
         unit /= np.linalg.norm(unit, axis=1, keepdims=True)
         errors.append(score.cpu().numpy() - (unit * unit[nn.cpu().numpy()]).sum(axis=1))
     assert np.sqrt(np.mean(np.square(errors))) <= rms
+
+
+@pytest.mark.parametrize("n", [64, 1500])
+def test_orthogonal_rows(mpm, n):
+    """Cosines of exactly 0 everywhere: every row's neighbour is the lowest other index, so only rows 0 and 1 pair up."""
+    x = torch.zeros(n, 1536, device=DEV)
+    x[torch.arange(n), torch.arange(n)] = 3.0
+    off = torch.tensor([0, n], device=DEV)
+    nn, score = mpm.nearest_neighbors(x, off)
+    assert nn.tolist() == [1] + [0] * (n - 1) and not score.any()
+    out, out_off, rmap = mpm.merge(x, off)
+    assert out_off.tolist() == [0, n - 1]
+    assert rmap.tolist() == [0, 0] + list(range(1, n - 1))
