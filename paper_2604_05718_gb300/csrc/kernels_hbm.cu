@@ -95,8 +95,12 @@ __device__ __forceinline__ int64_t warp_number(int block, int blocks, bool sprea
   return spread ? static_cast<int64_t>(w) * blocks + block : static_cast<int64_t>(block) * (kThreads / 32) + w;
 }
 
+// The blocks per SM are what the untraced kernel has anyway; asked for, the
+// traced library's kernels, with a few registers more, have them too.  (Without,
+// its pair average of 1.5 KiB rows kept two blocks an SM instead of three, and
+// its timeline said 26.4 us for what takes 22.  0 leaves a kernel as it is.)
 template <int ROWS, int VECS>
-__global__ void __launch_bounds__(kThreads) prep_kernel(const uint8_t* __restrict__ tokens,
+__global__ void __launch_bounds__(kThreads, VECS == 4 ? 0 : 5) prep_kernel(const uint8_t* __restrict__ tokens,
                                                         const int64_t* __restrict__ offsets,
                                                         int batch, int64_t rows, int row_bytes,
                                                         bool bf16, AffinityTile tile,
@@ -541,7 +545,7 @@ __device__ __noinline__ int scan_again(const float* tokens, int batch, int dim, 
 // block an SM only where the registers of four rows a thread and a cluster ask
 // for it.)
 template <int ELEMS, bool CLUSTER, bool SPLIT>
-__global__ void __launch_bounds__(kScanThreads, CLUSTER && ELEMS > 1 ? 1 : 2)
+__global__ void __launch_bounds__(kScanThreads, CLUSTER && ELEMS > 1 ? 0 : 2)
     mutual_compact_kernel(const float* __restrict__ tokens, int batch, int dim, int chunk, Workspace ws,
                           int32_t* __restrict__ out_map, int64_t* __restrict__ out_offsets) {
   MPM_TRACE_BEGIN(MPM_TRACE_MUTUAL);
@@ -681,7 +685,7 @@ __global__ void __launch_bounds__(kScanThreads, CLUSTER && ELEMS > 1 ? 1 : 2)
 // R consecutive output rows at a time, U vectors of each in flight per lane:
 // all loads of a pass are issued before any store.
 template <int U, int R, bool ONE>
-__global__ void __launch_bounds__(kThreads) pair_average_kernel(const uint8_t* __restrict__ tokens,
+__global__ void __launch_bounds__(kThreads, R == 1 ? 0 : 3) pair_average_kernel(const uint8_t* __restrict__ tokens,
                                                                 uint8_t* __restrict__ out,
                                                                 int batch, int64_t rows, int row_bytes,
                                                                 bool bf16, Workspace ws, int64_t* out_offsets,
