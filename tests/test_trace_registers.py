@@ -40,5 +40,5 @@ def test_traced_kernels_keep_their_blocks_per_sm(tmp_path):
     plain = registers(tmp_path / "plain.o", [])
     traced = registers(tmp_path / "traced.o", ["-DMPM_TRACE"])
     plain, traced = blocks_per_sm(plain), blocks_per_sm(traced)
-    assert len(plain) >= 20
+    assert len(plain) >= 15
     assert plain == traced
