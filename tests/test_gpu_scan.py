@@ -44,7 +44,8 @@ def mpm():
     ([3, 1, 2] * 400, 0),             # more images than a block has threads
     ([2] * 1024, 0),                  # the pair average adds up to 1024 counts itself
     ([2, 1, 0] * 341 + [3, 3], 0),    # 1025 images: the scan does
-    ([2300] * 80, 256),               # too many images for two blocks each
+    ([2300] * 80, 256),               # too many images for two blocks each, four rows a thread
+    ([2300] * 70, 256),               # few enough
     ([700], 1 << 40),                 # a chunk longer than any image
 ])
 def test_scan_equals_the_oracles_compaction(mpm, counts, chunk):
