@@ -131,6 +131,11 @@ struct Item {
   int narrow;    // 1: a 256 x 128 tile (N = 128 MMAs) of columns col0 .. col0 + 127
 };
 
+// The epilogue stores column results 16 bytes at a time into the scratch that
+// follows the items and the staged plan and offsets.
+static_assert(kMaxItems * sizeof(Item) % 16 == 0 && 2 * (kMaxStagedImages + 1) * sizeof(int64_t) % 16 == 0,
+              "scratch on a 16-byte boundary");
+
 template <int EPIW>
 constexpr size_t smem_bytes() {
   return 1024 + static_cast<size_t>(STAGES) * STAGE_BYTES + Epi<EPIW>::WARPS * Epi<EPIW>::COLS * sizeof(float) +
