@@ -44,6 +44,8 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 L2_FLUSH_BYTES = 256 << 20
 KERNELS_PER_MERGE = 4
+# Merges that take the mutual scan and the pair average in one launch
+# (merge_tail_fits in kernels_hbm.cu), unless stage events ask for two.
 SMALL_MERGE_ROWS, SMALL_MERGE_IMAGES = 1024, 256
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "affinity_pair_traffic.txt")
 # The sources the affinity kernel is compiled from; the traffic record holds
@@ -331,6 +333,18 @@ def new_events(stream, n):
     return evs
 
 
+def small_merge(rows: int, images: int) -> bool:
+    return rows <= SMALL_MERGE_ROWS and images <= SMALL_MERGE_IMAGES
+
+
+def kernel_times_of(rows: int, images: int) -> str:
+    """What the per-kernel durations describe, beside the timed step."""
+    if small_merge(rows, images):
+        return ("the two-launch merge that events between the kernels ask for; the timed step takes mutual scan and "
+                "pair average in one launch")
+    return "the timed step's kernels, with events between them"
+
+
 class StepEvents:
     """The CUDA events of one step."""
 
@@ -379,7 +393,7 @@ class Step:
 
     def launches(self) -> int:
         """Kernels of the library launched by one step (a merge of few rows takes its last two steps in one)."""
-        per_merge = KERNELS_PER_MERGE - (self.batch.rows <= SMALL_MERGE_ROWS and self.batch.batch <= SMALL_MERGE_IMAGES)
+        per_merge = KERNELS_PER_MERGE - small_merge(self.batch.rows, self.batch.batch)
         return 2 * per_merge + 1 if self.two else per_merge + 1
 
     def run(self, ev: StepEvents, host_in=None, host_out=None, per_kernel=False):
@@ -559,6 +573,7 @@ def workload_summary(p: Step, t: dict, m: dict) -> dict:
         "affinity_peak": ("bf16 dense" if p.cfg.dtype == "bf16" else
                           "fp16 dense (the bf16 rate); three fp16 products per term"),
         "affinity_us": {k: v for k, v in t["kern"].items() if k.startswith("affinity")},
+        "kernel_times_of": kernel_times_of(p.batch.rows, p.batch.batch),
         "pipeline_frac": m["pipeline"]["frac"],
     }
     out.update({k: v for k, v in m["hbm"].items() if k.endswith("_frac")})
@@ -867,7 +882,7 @@ def run_mpm(args):
             "padded_batch": padded,
             "chunked_similarity": chunked,
             "fp32_nearest_neighbours": fp32,
-            "kernels_us": kern,
+            "kernels_us": kern, "kernels_us_of": kernel_times_of(p.batch.rows, p.batch.batch),
             "ms_per_step_with_kernel_events": ms_with_kernel_events,
             "in_step": in_step,
             "cpu_baseline": cpu_base,

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import importlib.util
 import os
+import re
 
 import numpy as np
 import pytest
@@ -120,3 +121,24 @@ def test_workload_summary(bench):
     assert w["affinity_frac_of_burst"] == pytest.approx(m["aff_tflops"] / 1000.0, rel=1e-12)
     assert w["pipeline_frac"] == m["pipeline"]["frac"]
     assert w["pair_average_1_frac"] == m["hbm"]["pair_average_1_frac"]
+
+
+def test_small_merge_matches_the_library(bench):
+    """The launch count and the label of the per-kernel times follow the library's rule for one-launch tails."""
+    with open(os.path.join(ROOT, "paper_2604_05718_gb300", "csrc", "kernels_hbm.cu")) as f:
+        src = f.read()
+
+    def constant(name):
+        return re.search(rf"constexpr int {name} = ([^;]+);", src).group(1)
+
+    threads, elems = int(constant("kThreads")), int(constant("kTailElems"))
+    assert constant("kTailRows") == "kTailElems * kThreads" and constant("kTailImages") == "kThreads"
+    assert (bench.SMALL_MERGE_ROWS, bench.SMALL_MERGE_IMAGES) == (elems * threads, threads)
+    assert "return rows > 0 && rows <= kTailRows && batch <= kTailImages;" in src
+    assert bench.small_merge(1024, 256) and not bench.small_merge(1025, 1) and not bench.small_merge(300, 257)
+    step = bench.Step.__new__(bench.Step)
+    step.two = True
+    for rows, images, launches in ((1024, 1, 7), (65536, 64, 9)):
+        step.batch = type("B", (), {"rows": rows, "batch": images})
+        assert step.launches() == launches
+        assert ("one launch" in bench.kernel_times_of(rows, images)) == (launches == 7)
