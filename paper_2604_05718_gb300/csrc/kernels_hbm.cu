@@ -1,8 +1,9 @@
 // Bandwidth-bound MPM kernels: row norms (Eq. 1), the mutual check and
 // left-to-right representative scan (Algorithm 1 steps 4-6), the pair
 // average with compaction (Eq. 2), map composition (Eq. 3) and the gather
-// reconstruction (Eq. 4).  All token traffic moves in 16-byte vectors, one
-// warp per row; grids are sized from the SM count and loop over rows.
+// reconstruction (Eq. 4).  All token traffic moves in 16-byte vectors, by warps
+// that take one or a few rows at a time; grids are sized from the SM count and
+// the rows.
 #include <math.h>
 
 #include <type_traits>
@@ -179,9 +180,12 @@ __global__ void __launch_bounds__(kThreads, VECS == 4 ? 0 : 5) prep_kernel(const
 // inv_norm receives the scaled rows' inverse norms (the plain ones times the
 // inverse power of two), which undo the scale in the cosines.
 //
-// Against fp64, the cosines of 700 tokens of 64 to 16384 features (normal,
-// clustered, heavy-tailed, offset, one feature 300 times the others) are 1.2
-// to 2 times closer than through tf32 parts: half as many accumulations.
+// Against fp64, the rms error of the best cosines is 0.35 (64 features) to 0.70
+// (4) times that through tf32 parts, 0.64 at 768, and neither it nor the largest
+// error is larger for any of 17 row lengths from 4 to 2048 and seven
+// distributions (normal, clustered, heavy-tailed, offset, positive, rows of
+// any scale, one feature 300 times the others): half as many accumulations, in
+// an order that keeps small terms (affinity_pair.cu).
 //
 // Bound by HBM: 65536 rows of 768 take 201 MB in and 201 MB out, 64.6 us (the
 // two fp32-sized tf32 parts took 100.2).
@@ -470,7 +474,9 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanElems = 4;
 constexpr int kScanMaxCluster = 8;
 constexpr int kAgain = 1 << 30;  // in a block's count: its image has to be scanned again
-// Images whose counts every block of the pair average adds up itself.
+// Images whose counts every block of the pair average adds up itself.  (Up to 256
+// only: merges of 257 x 64 x 64 rows 22.4 instead of 20.3 us, of 1024 x 64 x 64
+// 52.6 instead of 47.9, of 1024 x 150 x 384 116.3 instead of 106.4.)
 constexpr int kStagedImages = 1024;
 
 __device__ __forceinline__ uint32_t scan_cluster_rank() {
@@ -1005,14 +1011,14 @@ __global__ void compose_kernel(const int32_t* map1, const int64_t* __restrict__ 
 // Gather reconstruction (Eq. 4), a pure copy.  A warp takes `per_warp` (at
 // most kGatherRows) consecutive grid rows: lane l resolves row p0 + l (its
 // image, its map entry and the source row, all independent loads across the
-// lanes), then the warp copies the rows as one run of 16-byte vectors, U of
-// them in flight per lane whatever the row length.  With COMPOSE the source
+// lanes), then the warp copies the rows as one run of 16-byte vectors, up to U
+// of them in flight per lane (8 rows of less than 768 B have fewer).  With COMPOSE the source
 // is composed on the way (Eq. 3): r*(p) = map2[off1_b + map1[p]], and r* is
 // written to out_map if given.
 //
 // Large grids are bound by HBM, small ones by the chain of dependent loads
 // (offsets, maps, row), so the rows are dealt evenly over the whole GPU: 32
-// rows a warp, four at a time, left 1024 rows of 768 bf16 on 32 warps (10.0
+// rows a warp, four at a time, left 1024 rows of 192 fp32 on 32 warps (10.0
 // us, now 1.4) and 36864 rows of 1024 on 1152 warps (24.5 us, now 15.7).
 // Runs of 8 rows with 12 vectors in flight were the fastest on 65536 rows of
 // 768 bf16 (whole step 202.4 us; 4 rows and 8 vectors 203.3, up to 32 rows
@@ -1065,8 +1071,9 @@ struct ImageCursor {
 // Images from which on every block copies their offsets to shared memory: a
 // search in global memory is a chain of dependent loads (64 images of 1024 x
 // 768 bf16: 22.9 instead of 21.6 us, 32 of 1024 x 384: 8.1 instead of 7.5),
-// but for a few images the copy and its barrier take longer (3 images: 1.7
-// against 2.0 us).  The upper bound keeps the copy within 6 KiB.
+// but for a few images the copy and its barrier take longer (3 images of 1024 x
+// 384: 2.69 against 2.49 us; from 4 to 10 images the two are within 3%, 12: 3.75
+// against 3.85).  The upper bound keeps the copy within 6 KiB.
 constexpr int kStagedFrom = 9, kStagedTo = 256;
 
 template <int U, bool COMPOSE, bool STAGED>
