@@ -38,6 +38,10 @@ __device__ __forceinline__ void write_plan(const int64_t* __restrict__ offsets, 
   __shared__ int64_t sh[32];
   __shared__ int64_t ends[kThreads + 1];
   __shared__ int bad;
+  // The first images' offsets are on their way while the block meets.
+  const int tid = static_cast<int>(threadIdx.x), ahead = tid < batch ? tid : batch - 1;
+  const int64_t final_offset = offsets[batch];
+  int64_t raw = offsets[ahead + 1], prev = offsets[ahead];
   if (threadIdx.x == 0) {
     ws.status[0] = 0;
     ws.status[1] = 0;
@@ -45,14 +49,17 @@ __device__ __forceinline__ void write_plan(const int64_t* __restrict__ offsets, 
     bad = -1;
   }
   __syncthreads();
-  const int64_t used = clamp64(offsets[batch], 0, rows);
+  const int64_t used = clamp64(final_offset, 0, rows);
   int64_t acc = 0;
   for (int base = 0; base < batch; base += kThreads) {
     // Image `idx`: from soff[idx], which the thread before has, to soff[idx + 1].
-    const int idx = base + threadIdx.x;
+    const int idx = base + tid;
     int64_t end = 0;
     if (idx < batch) {
-      const int64_t raw = offsets[idx + 1], prev = offsets[idx];
+      if (base > 0) {
+        raw = offsets[idx + 1];
+        prev = offsets[idx];
+      }
       if (raw < prev || raw > rows) atomicCAS(&bad, -1, idx + 1);
       end = clamp64(raw, 0, used);
       if (idx == 0) {
@@ -857,11 +864,13 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
   const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
   int j[kTailElems], image[kTailElems];
   [[maybe_unused]] bool redo = false;
+  // Rows of the capacity past the last image have no keys of this call.
+  [[maybe_unused]] const int64_t used_rows = SPLIT ? ws.soff[batch] : 0;
 #pragma unroll
   for (int e = 0; e < kTailElems; ++e) {
     const int i = e * kThreads + tid;
     const unsigned long long key = i < rows ? ws.keys[i] : 0ull;
-    if (SPLIT) redo |= maybe_undecided(key);
+    if (SPLIT) redo |= maybe_undecided(key) & (i < used_rows);
     j[e] = key_index(key);
   }
   for (int idx = tid; idx <= batch; idx += kThreads) first_s[idx] = static_cast<int32_t>(ws.soff[idx]);

@@ -236,3 +236,21 @@ def test_orthogonal_rows(mpm, n):
     out, out_off, rmap = mpm.merge(x, off)
     assert out_off.tolist() == [0, n - 1]
     assert rmap.tolist() == [0, 0] + list(range(1, n - 1))
+
+
+def test_capacity_past_the_last_image_changes_nothing(mpm):
+    """Small merges with spare rows: what the workspace holds for those is nobody's key, whatever it looks like."""
+    rng = np.random.default_rng(2)
+    x = torch.zeros(300, 64)
+    x[:100] = torch.from_numpy(rng.standard_normal((100, 64)).astype(np.float32))
+    xd, off = x.to(DEV), torch.tensor([0, 60, 100], device=DEV)
+    results = []
+    for fill in (0, 0x7F, 0x80, 0xFF):
+        ws = mpm.new_workspace(300, 2, 64, xd.dtype, DEV)
+        ws.fill_(fill)
+        out, rmap = torch.full_like(xd, 7.0), torch.full((300,), -5, dtype=torch.int32, device=DEV)
+        _, out_off, _ = mpm.merge(xd, off, workspace=ws, out_tokens=out, out_map=rmap)
+        assert mpm.device_status(ws) == 0
+        results.append((out, out_off, rmap))
+    for r in results[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(results[0], r))
