@@ -1209,8 +1209,14 @@ cudaError_t launch_prep(const void* tokens, const int64_t* offsets, int batch, i
   // Rows and vectors per warp and round by the row's length, so that no load
   // slot is empty: with 2 x 3 for every length, rows of 2 KiB took two passes
   // (36864 of them 17.9 us, now 16.5) and rows of 768 B half the slots (32768
-  // of them 8.7, now 8.0); 4 x 3 and 1 x 3 were slower for 1.5 KiB.
+  // of them 8.7, now 8.0); 4 x 3 and 1 x 3 were slower for 1.5 KiB.  Rows of
+  // 2 to 6 KiB take the width that their passes fill better: 3 for 1152, 1232 and
+  // 2144 features (queries of 64-token images 43.1 instead of 45.2 us, 41.7
+  // instead of 42.9, 39.1 instead of 40.7), 4 for 1544 and 2048 (51.9 instead of
+  // 52.6, 36.6 instead of 36.9) and for longer rows (3584: 40.0 instead of 40.7).
   const int nvec = row_bytes >> 4;
+  const bool three =
+      nvec > 64 && (nvec <= 96 || (nvec > 128 && nvec <= 384 && (nvec + 95) / 96 * 96 <= (nvec + 127) / 128 * 128));
   const auto launch = [&](auto kernel, int per_sm, int warp_rows) {
     const RowGrid g = row_grid((rows + warp_rows - 1) / warp_rows, grid_for(num_sms, per_sm) - 1);
     return launch_dependent(kernel, dim3(1 + g.blocks), dim3(kThreads), 0, stream, static_cast<const uint8_t*>(tokens),
@@ -1224,7 +1230,7 @@ cudaError_t launch_prep(const void* tokens, const int64_t* offsets, int batch, i
     static const int per_sm = resident_per_sm(prep_kernel<3, 2>, kThreads, 8);
     return launch(prep_kernel<3, 2>, per_sm, 3);
   }
-  if (nvec <= 96) {
+  if (three) {
     static const int per_sm = resident_per_sm(prep_kernel<2, 3>, kThreads, 8);
     return launch(prep_kernel<2, 3>, per_sm, 2);
   }

@@ -40,6 +40,9 @@ def mpm():
     ("bf16", 776, [130], 0),                  # 97
     ("bf16", 1024, [31, 31], 0),              # 128
     ("bf16", 1032, [50], 2),                  # 129: two passes
+    ("bf16", 1536, [41], 0),                  # 192: two full passes of three vectors
+    ("bf16", 1544, [41], 0),                  # 193: two passes of four
+    ("bf16", 2056, [33], 1),                  # 257: three of three
     ("f32", 2052, [45, 1], 0),                # 513
     ("bf16", 16, [5] * 255, 0),               # as many images as the plan's block has threads, and one more
     ("bf16", 16, [5] * 256, 0),
