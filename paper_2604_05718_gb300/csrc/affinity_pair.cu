@@ -738,8 +738,8 @@ cudaError_t launch_affinity_pair(const void* tokens, int batch, int64_t rows, in
   if (encode == nullptr) return cudaErrorNotSupported;
   // bf16: the tokens themselves; fp32: the fp16 high and low parts that the
   // prep kernel wrote into the workspace.
-  const cuuint64_t gdim[2] = {static_cast<cuuint64_t>(dim), static_cast<cuuint64_t>(rows)};
-  const cuuint64_t gstride[1] = {static_cast<cuuint64_t>(split ? split_stride(dim) : dim) * 2};
+  const cuuint64_t gdim[2] = {static_cast<cuuint64_t>(split ? split_stride(dim) : dim), static_cast<cuuint64_t>(rows)};
+  const cuuint64_t gstride[1] = {gdim[0] * 2};
   const cuuint32_t box[2] = {BOX_K, HALF};
   const cuuint32_t estride[2] = {1, 1};
   const CUtensorMapDataType type = split ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;

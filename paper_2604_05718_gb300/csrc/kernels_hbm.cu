@@ -197,8 +197,6 @@ __global__ void __launch_bounds__(kThreads, VECS == 4 ? 0 : 5) prep_kernel(const
 // Bound by HBM: 65536 rows of 768 take 201 MB in and 201 MB out, 64.6 us (the
 // two fp32-sized tf32 parts took 100.2).
 // ---------------------------------------------------------------------------
-constexpr int kSplitVecs = 8;  // 16-byte vectors of a row that a lane keeps in registers (D <= 1024)
-
 struct RowScale {
   float s1, s2;  // the row's scale is s1 * s2
   float inv;     // 1 / max(|x|, 1e-12) of the scaled row
@@ -264,6 +262,9 @@ __device__ __forceinline__ RowScale row_scale(const uint4* src, int nvec, float 
           1.0f / fmaxf(norm, 1e-12f) * __uint_as_float(static_cast<uint32_t>(127 - e) << 23)};
 }
 
+// ROWS rows a warp and round, VECS 16-byte vectors of each in registers; with
+// one row, further vectors of a longer row are read twice.
+template <int ROWS, int VECS>
 __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __restrict__ tokens,
                                                               const int64_t* __restrict__ offsets, int batch,
                                                               int64_t rows, int dim, AffinityTile tile,
@@ -282,44 +283,60 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
   const int64_t warp = warp_number(blockIdx.x - 1, gridDim.x - 1, spread);
   const int64_t nwarps = static_cast<int64_t>(gridDim.x - 1) * (kThreads / 32);
   const int nvec = dim >> 2;
-  const int64_t stride = split_stride(dim) >> 2;  // in groups of four values
-  for (int64_t g = warp; g < used; g += nwarps) {
-    const int64_t r = used - 1 - g;  // last row first, as in prep_kernel
-    const uint4* src = reinterpret_cast<const uint4*>(tokens) + r * nvec;
-    uint4 buf[kSplitVecs];
-    float s = 0.f;
+  const int stride = split_stride(dim) >> 2;  // in groups of four values; those past nvec are zeros
+  for (int64_t g0 = warp * ROWS; g0 < used; g0 += nwarps * ROWS) {
+    const int64_t r0 = used - 1 - g0;  // last row first, as in prep_kernel
+    const uint4* const src0 = reinterpret_cast<const uint4*>(tokens) + r0 * nvec;
+    uint4 buf[ROWS][VECS];
+    float s[ROWS];
 #pragma unroll
-    for (int u = 0; u < kSplitVecs; ++u) {
-      const int v = lane + 32 * u;
-      buf[u] = v < nvec ? __ldg(src + v) : make_uint4(0, 0, 0, 0);
-    }
+    for (int k = 0; k < ROWS; ++k)
 #pragma unroll
-    for (int u = 0; u < kSplitVecs; ++u) s += sumsq16(buf[u], false);
-    for (int v = lane + 32 * kSplitVecs; v < nvec; v += 32) s += sumsq16(__ldg(src + v), false);
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
-    const RowScale sc = row_scale(src, nvec, s);
-    uint2* hi = reinterpret_cast<uint2*>(ws.split_hi) + r * stride;
-    uint2* lo = reinterpret_cast<uint2*>(ws.split_lo) + r * stride;
-#pragma unroll
-    for (int u = 0; u < kSplitVecs; ++u) {
-      const int v = lane + 32 * u;
-      if (v < nvec) {
-        uint2 h, l;
-        split_f16(buf[u], sc.s1, sc.s2, h, l);
-        hi[v] = h;
-        lo[v] = l;
+      for (int u = 0; u < VECS; ++u) {
+        const int v = lane + 32 * u;
+        buf[k][u] = (v < nvec && g0 + k < used) ? __ldg(src0 - k * nvec + v) : make_uint4(0, 0, 0, 0);
       }
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k) {
+      s[k] = 0.f;
+#pragma unroll
+      for (int u = 0; u < VECS; ++u) s[k] += sumsq16(buf[k][u], false);
     }
-    for (int v = lane + 32 * kSplitVecs; v < nvec; v += 32) {
-      uint2 h, l;
-      split_f16(__ldg(src + v), sc.s1, sc.s2, h, l);
-      hi[v] = h;
-      lo[v] = l;
+    if (ROWS == 1)
+      for (int v = lane + 32 * VECS; v < nvec; v += 32) s[0] += sumsq16(__ldg(src0 + v), false);
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k) {
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], d);
     }
-    if (lane == 0) {
-      ws.inv_norm[r] = sc.inv;
-      ws.keys[r] = 0ull;
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k) {
+      if (g0 + k >= used) break;
+      const int64_t r = r0 - k;
+      const RowScale sc = row_scale(src0 - k * nvec, nvec, s[k]);
+      uint2* hi = reinterpret_cast<uint2*>(ws.split_hi) + r * stride;
+      uint2* lo = reinterpret_cast<uint2*>(ws.split_lo) + r * stride;
+#pragma unroll
+      for (int u = 0; u < VECS; ++u) {
+        const int v = lane + 32 * u;
+        if (v < stride) {
+          uint2 h, l;
+          split_f16(buf[k][u], sc.s1, sc.s2, h, l);
+          hi[v] = h;
+          lo[v] = l;
+        }
+      }
+      if (ROWS == 1)
+        for (int v = lane + 32 * VECS; v < stride; v += 32) {
+          uint2 h, l;
+          split_f16(v < nvec ? __ldg(src0 + v) : make_uint4(0, 0, 0, 0), sc.s1, sc.s2, h, l);
+          hi[v] = h;
+          lo[v] = l;
+        }
+      if (lane == 0) {
+        ws.inv_norm[r] = sc.inv;
+        ws.keys[r] = 0ull;
+      }
     }
   }
 }
@@ -1201,10 +1218,31 @@ cudaError_t launch_prep(const void* tokens, const int64_t* offsets, int batch, i
                         cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
   if (ws.split_hi != nullptr) {
-    static const int per_sm = resident_per_sm(prep_split_kernel, kThreads, 8);
-    const RowGrid g = row_grid(rows, grid_for(num_sms, per_sm) - 1);
-    return launch_dependent(prep_split_kernel, dim3(1 + g.blocks), dim3(kThreads), 0, stream,
-                            static_cast<const uint8_t*>(tokens), offsets, batch, rows, dim, tile, ws, g.spread);
+    const auto launch = [&](auto kernel, int per_sm, int warp_rows) {
+      const RowGrid g = row_grid((rows + warp_rows - 1) / warp_rows, grid_for(num_sms, per_sm) - 1);
+      return launch_dependent(kernel, dim3(1 + g.blocks), dim3(kThreads), 0, stream,
+                              static_cast<const uint8_t*>(tokens), offsets, batch, rows, dim, tile, ws, g.spread);
+    };
+    // Rows and vectors per warp and round by the row's length, in as few
+    // registers as it needs.  One row and eight vectors for every length left most
+    // slots of short rows empty: queries of 64-token images, 3000 of 16 features
+    // 104.8 us (75.5 with 2 x 1, 82.0 with 1 x 1, 78.1 with 4 x 1), 976 of 192 features
+    // 59.1 (50.0 with 2 x 2, 50.7 with 1 x 2), 488 of 384 49.2 (47.2 with 1 x 4, 48.3
+    // with 2 x 4).
+    if (dim <= 128) {
+      static const int per_sm = resident_per_sm(prep_split_kernel<2, 1>, kThreads, 8);
+      return launch(prep_split_kernel<2, 1>, per_sm, 2);
+    }
+    if (dim <= 256) {
+      static const int per_sm = resident_per_sm(prep_split_kernel<2, 2>, kThreads, 8);
+      return launch(prep_split_kernel<2, 2>, per_sm, 2);
+    }
+    if (dim <= 512) {
+      static const int per_sm = resident_per_sm(prep_split_kernel<1, 4>, kThreads, 8);
+      return launch(prep_split_kernel<1, 4>, per_sm, 1);
+    }
+    static const int per_sm = resident_per_sm(prep_split_kernel<1, 8>, kThreads, 8);
+    return launch(prep_split_kernel<1, 8>, per_sm, 1);
   }
   // Rows and vectors per warp and round by the row's length, so that no load
   // slot is empty: with 2 x 3 for every length, rows of 2 KiB took two passes

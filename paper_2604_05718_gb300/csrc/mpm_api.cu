@@ -40,8 +40,8 @@ struct Layout {
 };
 
 // split_elems: rows * dim for fp32 tokens, 0 for bf16.  Each split part is
-// given 4 bytes per element, twice what its fp16 values take (rows padded to
-// 8 values included): the documented workspace size, which also decides what
+// given 4 bytes per element, which holds its fp16 rows (2 split_stride(dim) <=
+// 4 dim bytes each): the documented workspace size, which also decides what
 // mpm_merge_no_alloc accepts.
 Layout layout(int64_t rows, int32_t batch, size_t split_elems) {
   Layout l{};

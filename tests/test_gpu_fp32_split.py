@@ -52,12 +52,29 @@ def check(mpm, x: np.ndarray, rows=None):
     assert np.all(s[rows].max(axis=1) - chosen <= 2 * tol)
 
 
-@pytest.mark.parametrize("dim", [4, 8, 12, 60, 68, 196, 1024, 1028, 4100])
+@pytest.mark.parametrize("dim", [4, 8, 12, 60, 68, 128, 132, 196, 256, 260, 512, 516, 1024, 1028, 4100])
 def test_row_lengths(mpm, dim):
     rng = np.random.default_rng(dim)
     means = rng.standard_normal((9, dim))
     x = means[rng.integers(0, 9, 300)] + 0.3 * rng.standard_normal((300, dim))
     check(mpm, x.astype(np.float32))
+
+
+@pytest.mark.parametrize("dim", [8, 100, 132])
+def test_non_finite_rows_that_are_padded(mpm, dim):
+    """Rows whose fp16 parts end in padding: a row with a NaN or an infinity spoils no other row's cosines."""
+    rng = np.random.default_rng(dim)
+    x = (rng.standard_normal((77, dim)) + 1.0).astype(np.float32)
+    x[20, dim - 1] = np.nan
+    x[76, 0] = np.inf
+    nn, score = (t.cpu().numpy() for t in mpm.nearest_neighbors(torch.from_numpy(x).to(DEV),
+                                                                torch.tensor([0, 77], device=DEV)))
+    good = np.setdiff1d(np.arange(77), [20, 76])
+    assert nn[20] == nn[76] == -1 and not np.isin(nn[good], [20, 76]).any()
+    s = oracle.cosine_affinity(x[good].astype(np.float64))
+    chosen = s[np.arange(75), np.searchsorted(good, nn[good])]
+    np.testing.assert_allclose(score[good], chosen, rtol=0, atol=bound(dim))
+    assert np.all(s.max(axis=1) - chosen <= 2 * bound(dim))
 
 
 def test_rows_of_any_magnitude(mpm):
