@@ -84,7 +84,7 @@ typedef enum mpm_nn_algo {
                               term (a row's values scaled by one power of two,
                               x = hi + lo with hi the fp16 rounding of x:
                               hi.hi + hi.lo + lo.hi, accumulated in fp32;
-                              rows whose best cosine is below 2^-15 in size
+                              rows whose best cosine is below 2^-16 in size
                               are decided by fp32 products of the tokens) */
 } mpm_nn_algo;
 

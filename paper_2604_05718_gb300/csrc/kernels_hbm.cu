@@ -359,14 +359,15 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
 // 4096 x 768, and as long again for each further such row.
 // ---------------------------------------------------------------------------
 // Is the row's best cosine too small to trust?  Its score is the cosine times
-// the scaled row's norm, 2^14 to 2^15: above 1 it needs no look at the norm.
+// the scaled row's norm, 2^14 to 2^15 (whatever the norm's floor makes of the row
+// itself), so that this holds below 2^-16 and never above 2^-15.
+__device__ __forceinline__ bool undecided(unsigned long long key) {
+  return (key != 0ull) & (fabsf(key_score(key)) < 0.5f);
+}
 // Zero rows, whose cosines are exactly 0, need nothing: their inverse norm is
 // 1e12, every other row's, scaled, at most 2^-7 or so.
-__device__ __forceinline__ bool maybe_undecided(unsigned long long key) {
-  return (key != 0ull) & (fabsf(key_score(key)) < 1.0f);
-}
 __device__ __forceinline__ bool undecided(unsigned long long key, float inv_norm) {
-  return (key != 0ull) & (inv_norm < 1e11f) & (fabsf(key_score(key) * inv_norm) < 0x1p-15f);
+  return undecided(key) & (inv_norm < 1e11f);
 }
 
 // Does any of the rows r0 .. r1 - 1 have an element that its parts do not hold to
@@ -406,11 +407,14 @@ __device__ __noinline__ bool any_cut_element(const float* __restrict__ tokens, i
 // the neighbour's scaled inverse norm.  Ties go to the lowest index and NaN
 // never wins.  Scores are compared 2^96 times as large (at most 2^126), so that
 // products of two rows' smallest features do not vanish.  Called by all threads
-// of a block: one row at a time, its candidates dealt over the warps.
+// of a block: one row at a time, its candidates dealt over the warps.  A score
+// that is small because the best neighbour's norm is below the floor (the errors
+// are as much smaller) stays as it is.
 __device__ __noinline__ unsigned long long decide(bool redo, unsigned long long key, int64_t row,
                                                   const float* __restrict__ tokens, int dim, int batch, int chunk,
-                                                  const int64_t* soff) {
+                                                  const int64_t* soff, const float* inv_norm) {
   __shared__ unsigned long long turn, best;  // the next row (and its thread below it); its best key
+  __shared__ bool floored;
   const int lane = threadIdx.x & 31, nvec = dim >> 2;
   const auto sum = [](float s) {
 #pragma unroll
@@ -452,6 +456,16 @@ __device__ __noinline__ unsigned long long decide(bool redo, unsigned long long 
     const int n = static_cast<int>(soff[b + 1] - base), local = static_cast<int>(r - base);
     const int first = chunk > 0 ? (local / chunk) * chunk : 0;
     const int end = chunk > 0 && n - first > chunk ? first + chunk : n;
+    if (mine == now) {
+      // Without the floor, 1 / 2^15 < inv_norm.
+      const float inv_j = inv_norm[base + key_index(key)];
+      floored = inv_j < 0.99f * 0x1p-15f && fabsf(key_score(key)) >= 0.5f * 0x1p15f * inv_j;
+    }
+    __syncthreads();
+    if (floored) {
+      redo = redo && mine != now;
+      continue;
+    }
     const uint4* const rows = reinterpret_cast<const uint4*>(tokens);
     const uint4* const x = rows + r * nvec;
     const RowScale a = row_scale(x, nvec, products(x, x, 1.f, 1.f, 1.f, 1.f).x);
@@ -539,7 +553,7 @@ __device__ __forceinline__ bool neighbour_ok(int j, int i, int n, int chunk) {
 // returns the number of representatives.
 __device__ __noinline__ int scan_again(const float* tokens, int batch, int dim, int chunk, const int64_t* soff,
                                        const unsigned long long* keys, const float* inv_norm, int b, int32_t* out_map,
-                                       int2* out_reps) {
+                                       int2* out_reps, int32_t* status) {
   __shared__ int32_t sh[32];
   const int64_t base = soff[b];
   const int n = static_cast<int>(soff[b + 1] - base);
@@ -549,11 +563,16 @@ __device__ __noinline__ int scan_again(const float* tokens, int batch, int dim, 
     const int i = c0 + static_cast<int>(threadIdx.x);
     const bool live = i < n;
     unsigned long long key = live ? keys[base + i] : 0ull;
-    key = decide(cut && live && undecided(key, inv_norm[base + i]), key, base + i, tokens, dim, batch, chunk, soff);
+    key = decide(cut && live && undecided(key, inv_norm[base + i]), key, base + i, tokens, dim, batch, chunk, soff,
+                 inv_norm);
     int j = key_index(key);
-    if (!live || !neighbour_ok(j, i, n, chunk)) j = -1;
+    if (live && !neighbour_ok(j, i, n, chunk)) {
+      report(status, MPM_ERR_DEVICE_CHECK, static_cast<int32_t>(base + i));
+      j = -1;
+    }
     key = j >= 0 ? keys[base + j] : 0ull;
-    key = decide(cut && j >= 0 && undecided(key, inv_norm[base + j]), key, base + j, tokens, dim, batch, chunk, soff);
+    key = decide(cut && j >= 0 && undecided(key, inv_norm[base + j]), key, base + j, tokens, dim, batch, chunk, soff,
+                 inv_norm);
     if (key_index(key) != i) j = -1;
     const bool rep = live && (j < 0 || i < j);
     int total;
@@ -609,7 +628,7 @@ __global__ void __launch_bounds__(kScanThreads, CLUSTER && ELEMS > 1 ? 0 : 2)
     for (int e = 0; e < ELEMS; ++e) {
       const int64_t i = first + e * kScanThreads;
       const unsigned long long key = (e < elems && i < n) ? ws.keys[base + i] : 0ull;
-      if (SPLIT) redo |= maybe_undecided(key);
+      if (SPLIT) redo |= undecided(key);
       j[e] = key_index(key);
     }
 #pragma unroll
@@ -624,7 +643,7 @@ __global__ void __launch_bounds__(kScanThreads, CLUSTER && ELEMS > 1 ? 0 : 2)
         // (i, j) is a pair of P when b(j) = i as well (Section 3.2).
         if (j[e] >= 0) {
           const unsigned long long key = ws.keys[base + j[e]];
-          if (SPLIT) redo |= maybe_undecided(key);
+          if (SPLIT) redo |= undecided(key);
           if (key_index(key) != i) j[e] = -1;
         }
         rep = j[e] < 0 || i < j[e];
@@ -682,7 +701,7 @@ __global__ void __launch_bounds__(kScanThreads, CLUSTER && ELEMS > 1 ? 0 : 2)
   }
   if (rank != 0) return;
   if (SPLIT && again)
-    carry = scan_again(tokens, batch, dim, chunk, ws.soff, ws.keys, ws.inv_norm, b, out_map, ws.reps);
+    carry = scan_again(tokens, batch, dim, chunk, ws.soff, ws.keys, ws.inv_norm, b, out_map, ws.reps, ws.status);
   if (threadIdx.x == 0) ws.count[b] = carry;
   if (batch <= kStagedImages) return;
   // More images than the pair average's blocks turn into offsets themselves:
@@ -887,7 +906,7 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
   for (int e = 0; e < kTailElems; ++e) {
     const int i = e * kThreads + tid;
     const unsigned long long key = i < rows ? ws.keys[i] : 0ull;
-    if (SPLIT) redo |= maybe_undecided(key) & (i < used_rows);
+    if (SPLIT) redo |= undecided(key) & (i < used_rows);
     j[e] = key_index(key);
   }
   for (int idx = tid; idx <= batch; idx += kThreads) first_s[idx] = static_cast<int32_t>(ws.soff[idx]);
@@ -902,7 +921,8 @@ __global__ void __launch_bounds__(kThreads) merge_tail_kernel(const uint8_t* __r
       const bool live = i >= lead && i < used;
       const unsigned long long key = live ? ws.keys[i] : 0ull;
       const int again = key_index(decide(cut && live && undecided(key, ws.inv_norm[i]), key, i,
-                                         reinterpret_cast<const float*>(tokens), row_bytes >> 2, batch, chunk, ws.soff));
+                                         reinterpret_cast<const float*>(tokens), row_bytes >> 2, batch, chunk, ws.soff,
+                                         ws.inv_norm));
 #pragma unroll
       for (int k = 0; k < kTailElems; ++k) j[k] = k == e && live ? again : j[k];
     }
@@ -991,12 +1011,12 @@ __global__ void __launch_bounds__(kThreads, 4) decode_nn_kernel(const float* __r
     const int64_t g = b0 + threadIdx.x;
     unsigned long long k = g < used ? ws.keys[g] : 0ull;
     const float inv = g < used ? ws.inv_norm[g] : 0.f;
-    if (SPLIT && __syncthreads_or(maybe_undecided(k))) {
+    if (SPLIT && __syncthreads_or(undecided(k))) {
       // The rows of all images that this block's rows belong to.
       const int64_t last = b0 + kThreads < used ? b0 + kThreads - 1 : used - 1;
       const int64_t r0 = ws.soff[find_image(ws.soff, batch, b0)], r1 = ws.soff[find_image(ws.soff, batch, last) + 1];
       if (any_cut_element(tokens, dim, r0, r1))
-        k = decide(undecided(k, inv), k, g, tokens, dim, batch, chunk, ws.soff);
+        k = decide(undecided(k, inv), k, g, tokens, dim, batch, chunk, ws.soff, ws.inv_norm);
     }
     if (g >= used) continue;
     nn[g] = key_index(k);

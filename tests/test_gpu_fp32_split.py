@@ -271,3 +271,37 @@ def test_capacity_past_the_last_image_changes_nothing(mpm):
         results.append((out, out_off, rmap))
     for r in results[1:]:
         assert all(torch.equal(a, b) for a, b in zip(results[0], r))
+
+
+def test_bad_rows_after_an_undecided_one_are_reported(mpm):
+    """A long image among short ones is scanned in rounds; one undecided row in the first must not hide a row without
+    a neighbour (here a NaN) in a later one."""
+    rng = np.random.default_rng(9)
+    counts = [5000] + [4] * 200
+    x = rng.standard_normal((sum(counts), 16)).astype(np.float32)
+    x[:, 0] = 0.0
+    x[3, 0] = 2.0 ** 60
+    off = torch.from_numpy(np.cumsum([0] + counts)).to(DEV)
+    ws = mpm.new_workspace(len(x), len(counts), 16, torch.float32, DEV)
+    for bad in (None, 4000, 3500):
+        xd = torch.from_numpy(x).to(DEV)
+        if bad is not None:
+            xd[bad, 2] = float("nan")
+        nn, _ = mpm.nearest_neighbors(xd, off, chunk=256)
+        out, out_off, rmap = mpm.merge(xd, off, workspace=ws, chunk=256)
+        assert mpm.device_status(ws) == (0 if bad is None else 6)
+        part, nn = rmap[:5000].cpu().numpy(), nn[:5000].cpu().numpy()
+        assert np.array_equal(part, oracle.compact_map(oracle.mutual_partners(nn))[0])
+
+
+def test_images_of_tiny_rows(mpm):
+    """Norms far below the floor of 1e-12: cosines scale with the neighbour's norm, in the oracle as here."""
+    rng = np.random.default_rng(6)
+    x = (rng.standard_normal((12, 48))[rng.integers(0, 12, 400)] + 0.3 * rng.standard_normal((400, 48))) * 1e-20
+    x = x.astype(np.float32)
+    nn, score = (t.cpu().numpy() for t in mpm.nearest_neighbors(torch.from_numpy(x).to(DEV),
+                                                                torch.tensor([0, 400], device=DEV)))
+    s = oracle.cosine_affinity(x.astype(np.float64))
+    chosen = s[np.arange(400), nn]
+    np.testing.assert_allclose(score, chosen, rtol=bound(48), atol=0)
+    assert np.all(s.max(axis=1) <= chosen * (1 + 2 * bound(48)))
