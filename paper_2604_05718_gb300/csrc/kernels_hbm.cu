@@ -344,8 +344,8 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
 // ---------------------------------------------------------------------------
 // fp32 rows that the fp16 parts cannot decide.  An element's parts are off by
 // at most 2^-39 of its row's norm (above): a cosine by about 2^-39 as the
-// errors' signs go, by 2^-39 sqrt(D) at worst.  A cosine of 2^-15 or more is
-// right to 2^-24, at worst 2^-24 sqrt(D), of its size, less than the products'
+// errors' signs go, by 2^-39 sqrt(D) at worst.  A cosine of 2^-16 or more is
+// right to 2^-23, at worst 2^-23 sqrt(D), of its size, no more than the products'
 // sum loses.  A row whose best cosine is smaller (rows with a huge feature of
 // their own: its other features decide, and may have lost bits or vanished)
 // has its neighbour found again by fp32 products of its run's tokens.  The
@@ -355,8 +355,8 @@ __global__ void __launch_bounds__(kThreads) prep_split_kernel(const uint8_t* __r
 // The check reads nothing that the kernels do not read anyway and costs 0.1 to
 // 0.5 us a merge (1024 x 192: 12.8 -> 13.0 us, 64 x 1024 x 192 80.9 -> 81.2, 64 x
 // 1024 x 384 117.0 -> 117.3); a kernel of its own before the scan cost 1.6 to 2.4.
-// Finding a row again takes one block: 0.12 ms among 1024 x 192, 0.19 ms among
-// 4096 x 768, and as long again for each further such row.
+// Finding a row again takes one block: 0.13 ms among 1024 x 192, 0.21 ms among
+// 4096 x 768, and about as long again for each further such row.
 // ---------------------------------------------------------------------------
 // Is the row's best cosine too small to trust?  Its score is the cosine times
 // the scaled row's norm, 2^14 to 2^15 (whatever the norm's floor makes of the row
