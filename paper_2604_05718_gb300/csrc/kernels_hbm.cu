@@ -1058,9 +1058,9 @@ __global__ void compose_kernel(const int32_t* map1, const int64_t* __restrict__ 
 // most kGatherRows) consecutive grid rows: lane l resolves row p0 + l (its
 // image, its map entry and the source row, all independent loads across the
 // lanes), then the warp copies the rows as one run of 16-byte vectors, up to U
-// of them in flight per lane (8 rows of less than 768 B have fewer).  With COMPOSE the source
-// is composed on the way (Eq. 3): r*(p) = map2[off1_b + map1[p]], and r* is
-// written to out_map if given.
+// of them in flight per lane.  With COMPOSE the source is composed on the way
+// (Eq. 3): r*(p) = map2[off1_b + map1[p]], and r* is written to out_map if
+// given.
 //
 // Large grids are bound by HBM, small ones by the chain of dependent loads
 // (offsets, maps, row), so the rows are dealt evenly over the whole GPU: 32
@@ -1071,8 +1071,25 @@ __global__ void compose_kernel(const int32_t* map1, const int64_t* __restrict__ 
 // and 8 vectors 203.6).
 // ---------------------------------------------------------------------------
 constexpr int kGatherVecs = 12;
-constexpr int kGatherRows = 8;
-static_assert(kGatherRows <= 32, "one lane resolves each row of a run");
+constexpr int kGatherRows = 32;  // one lane resolves each row of a run
+
+// Rows of `nvec` vectors per run, at most.  A grid that fits L2 takes runs of two
+// passes of a warp's vectors, 768, for rows shorter than 512 B, and 8 rows of
+// longer ones: 80 MB of rows of 128 B 17.8 us (with 8 rows 35.8), of 256 B 16.3
+// (21.7), 50 MB of rows of 768 B 10.4 us (with 16 rows 11.3).  A larger one is written fastest in runs of about 200 vectors, 3 KiB: 480
+// MB of rows of 1 KiB 112.9 us with 3 rows (126.8 with 8, 186.8 with 1), of 1.5 KiB
+// 113.1 with 2 (127.2), of 3 KiB 111.6 with 1 (127.8).  With 8 rows everywhere, rows of
+// 1, 1.25, 2 and 8 KiB were up to 6% slower there than with 32 rows a warp, four
+// at a time.
+int gather_rows(int64_t rows, int nvec) {
+  constexpr int64_t kLarge = 120'000'000;
+  int m;
+  if (rows * nvec * 16 > kLarge)
+    m = (200 + nvec / 2) / nvec;
+  else
+    m = nvec < 32 ? 2 * 32 * kGatherVecs / nvec : 8;
+  return m < 1 ? 1 : m < kGatherRows ? m : kGatherRows;
+}
 
 // Quotient e / nvec for 0 <= e < 2^17 and 1 <= nvec <= 2^12 (rows of at most
 // 64 KiB): magic = floor(2^31 / nvec) + 1, so the quotient is off by less than
@@ -1426,7 +1443,8 @@ cudaError_t launch_gather_kernel(const void* merged, const int64_t* moff, int64_
                                  int32_t* status, int num_sms, cudaStream_t stream) {
   const int row_bytes = dim * (bf16 ? 2 : 4);
   const auto launch = [&](auto kernel, int per_sm, size_t smem) {
-    const RunShape g = run_shape(grid_rows, grid_for(num_sms, per_sm), kThreads / 32, kGatherRows);
+    const RunShape g =
+        run_shape(grid_rows, grid_for(num_sms, per_sm), kThreads / 32, gather_rows(grid_rows, row_bytes >> 4));
     return launch_dependent(kernel, dim3(g.grid), dim3(kThreads), smem, stream, static_cast<const uint8_t*>(merged),
                             moff, merged_rows, map, goff, grid_rows, map2, off1, rows1, out_map, batch,
                             row_div(row_bytes), g.per_warp, static_cast<uint8_t*>(out), status);

@@ -1,6 +1,6 @@
 """Gather and fused compose + gather where their work split can go wrong.
 
-A warp copies a run of up to 8 grid rows as one sequence of 16-byte vectors,
+A warp copies a run of up to 32 grid rows as one sequence of 16-byte vectors,
 so the edges are: the shortest row (one vector), odd vector counts, the
 longest row, fewer rows than a run, runs that end within a warp's last load,
 and row counts around a whole round of warps.  The gather is a copy, so the
@@ -46,6 +46,11 @@ def offsets(counts):
     (torch.float32, 40, [0, 9, 0, 70, 1, 0, 33, 2, 500]),        # 9: from shared memory
     (torch.bfloat16, 8, [3] * 256),
     (torch.bfloat16, 8, [3, 1, 0] * 85 + [4, 5]),                # 257: in place again
+    (torch.bfloat16, 8, [200000, 77777]),          # several rounds of runs of 32 rows
+    (torch.bfloat16, 248, [700, 3, 29000]),        # 31 vectors: 24 rows, on the near side of the rule
+    (torch.bfloat16, 256, [700, 3, 29000]),        # 32: 8 rows
+    (torch.bfloat16, 512, [70000, 1, 50001]),      # more than 120 MB: runs of 3 rows
+    (torch.float32, 1540, [9000, 10600]),          # of one row
 ])
 def test_gather_equals_indexing(mpm, dtype, dim, counts):
     gen = torch.Generator(device=DEV).manual_seed(5)
